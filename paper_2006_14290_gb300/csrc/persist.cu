@@ -1,0 +1,170 @@
+// Host side of the single-launch solvers (persist.cuh): which systems they
+// take, the launch shape and the workspace.
+#include "persist.cuh"
+
+namespace gko {
+
+template <>
+PkKernel<double, double> pk_cg<double, double>(int, bool);
+template <>
+PkKernel<float, float> pk_cg<float, float>(int, bool);
+template <>
+PkKernel<float, __nv_bfloat16> pk_cg<float, __nv_bfloat16>(int, bool);
+template <>
+PkKernel<double, double> pk_bicg<double, double>(int, bool);
+template <>
+PkKernel<float, float> pk_bicg<float, float>(int, bool);
+template <>
+PkKernel<float, __nv_bfloat16> pk_bicg<float, __nv_bfloat16>(int, bool);
+
+namespace {
+
+// A matrix's column and value arrays in the formats served here.
+const Buf& cols_of(const gko_matrix_s* A) {
+  return A->fmt == GKO_CSR ? A->col : A->fmt == GKO_ELL ? A->ell_col : A->sellp_col;
+}
+const Buf& vals_of(const gko_matrix_s* A) {
+  return A->fmt == GKO_CSR ? A->val : A->fmt == GKO_ELL ? A->ell_val : A->sellp_val;
+}
+
+template <typename T, typename VT>
+int launch(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSpec& sp, cudaStream_t s, SolveOut* out,
+           int shape, bool staged, int G, size_t K, size_t smem) {
+  const int64_t n = A->n_rows;
+  const PkShape sh = kPkShapes[shape];
+  const bool cluster = sh.mode == kPkCluster;
+  const PkKernel<T, VT> kern = sp.solver == 0 ? pk_cg<T, VT>(shape, staged) : pk_bicg<T, VT>(shape, staged);
+  if (!kern) return GKO_NOT_SUPPORTED;
+  // always the largest request, so that concurrent solves (serving threads)
+  // never lower each other's limit
+  if (smem > 48 * 1024)
+    GKO_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPkSmemMax));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)G);
+  cfg.blockDim = dim3((unsigned)sh.nt);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (cluster) {
+    if (G > 8) GKO_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)G;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cluster) {
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) != cudaSuccess || fit < 1) {
+      cudaGetLastError();
+      return GKO_NOT_SUPPORTED;
+    }
+  }
+
+  const int nvec = cluster ? 0 : sp.solver == 0 ? (sh.mode == kPkFly ? 3 : 1) : (sh.mode == kPkFly ? 5 : 2);
+  const size_t slot_bytes = cluster ? 0 : sizeof(ulonglong2) * 2 * kPkMaxBlocks * kPkSlot;
+  Scratch mem;
+  GKO_TRY(mem.get(sizeof(Ctl) + slot_bytes + 1024 + (size_t)nvec * (sizeof(T) * (size_t)n + 320), s));
+  Carve cv{static_cast<char*>(mem.data())};
+  PkArgs<T, VT> a{};
+  a.n = (int32_t)n;
+  a.K = (int32_t)K;
+  a.fmt = A->fmt;
+  a.rp = A->fmt == GKO_CSR ? ptr<int32_t>(A->row_ptr) : A->fmt == GKO_SELLP ? ptr<int32_t>(A->sellp_sets) : nullptr;
+  a.col = ptr<int32_t>(cols_of(A));
+  a.val = ptr<VT>(vals_of(A));
+  a.stride = A->stride;
+  a.slice = A->slice;
+  a.b = b;
+  a.x = x;
+  a.d = static_cast<const T*>(sp.minv);
+  a.rel_tol = sp.rel_tol;
+  a.maxit = sp.maxit;
+  a.check_true = sp.check_true;
+  a.x_zero = x_zero ? 1 : 0;
+  if (sp.rel) {
+    a.val64 = ptr<double>(vals_of(sp.rel->A64));
+    a.b64 = sp.rel->b64;
+    a.x64 = sp.rel->x64;
+    a.delta = sp.rel->delta;
+  }
+  a.c = cv.take<Ctl>(1);
+  if (!cluster) a.slots = cv.take<ulonglong2>(2 * kPkMaxBlocks * kPkSlot);
+  for (int k = 0; k < nvec; ++k) a.vec[k] = cv.take<T>((size_t)n);
+  a.err = device_error_word();
+  if (!cluster) GKO_TRY_CUDA(cudaMemsetAsync(a.slots, 0, slot_bytes, s));
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {  // the blocks cannot all be resident
+    cudaGetLastError();
+    return GKO_NOT_SUPPORTED;
+  }
+  GKO_TRY_CUDA(e);
+  Ctl* hc = host_ctl();
+  GKO_TRY(read_ctl(a.c, hc, s));
+  if (hc->half) return fail(GKO_TIMEOUT, "single-launch solve: a grid reduction's wait timed out");
+  out->status = hc->status;
+  out->iterations = hc->iter;
+  out->cycles = hc->cycles;
+  if (sizeof(T) == 8) {
+    out->have_residual = true;
+    out->rel_residual = hc->nb == 0.0 ? 0.0 : sqrt(hc->rr) / hc->nb;
+  }
+  return GKO_OK;
+}
+
+template <typename T, typename VT>
+int run(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSpec& sp, cudaStream_t s,
+        SolveOut* out) {
+  const int64_t n = A->n_rows;
+  const size_t K = (size_t)std::max<int32_t>(1, A->fmt == GKO_CSR ? A->plan.max_len : A->K);
+  // the first shape that covers n and whose entries fit in shared memory;
+  // where none does, the first that reads its entries from the matrix
+  auto smem_of = [&](const PkShape& h, bool st) {
+    const size_t rb = (size_t)h.nt * h.rpt;
+    return (st ? K * rb * (sizeof(VT) + sizeof(int32_t)) : 0) + (h.mode == kPkCluster ? kPkClusterVecs * rb * sizeof(T) : 0);
+  };
+  auto blocks_of = [&](const PkShape& h) { return (n + h.nt * h.rpt - 1) / (h.nt * h.rpt); };
+  auto covers = [&](const PkShape& h) {
+    return blocks_of(h) <= (h.mode == kPkCluster ? kPkCluster16 : std::min(sm_count(), kPkMaxBlocks));
+  };
+  for (bool staged : {true, false})
+    for (int i = staged ? 0 : kPkFirstGlobal; i < kPkNShapes; ++i) {
+      if (!covers(kPkShapes[i]) || smem_of(kPkShapes[i], staged) > kPkSmemMax) continue;
+      const int rc = launch<T, VT>(A, b, x, x_zero, sp, s, out, i, staged, (int)blocks_of(kPkShapes[i]), K,
+                                   smem_of(kPkShapes[i], staged));
+      if (rc != GKO_NOT_SUPPORTED) return rc;
+    }
+  return GKO_NOT_SUPPORTED;
+}
+
+}  // namespace
+
+int persist_solve(const gko_matrix_s* A, const double* b, void* x, bool x_zero, const SolveSpec& sp, cudaStream_t s,
+                  SolveOut* out) {
+  // CSR under the row-block plan (regular rows: other plans keep their SpMV
+  // kernels), ELL and SELL-P; reliable updates for BiCGSTAB only
+  if (sp.solver > 1 || sp.bj || A->n_rows <= 0 || A->n_rows > kSmallRows) return GKO_NOT_SUPPORTED;
+  if (!(A->fmt == GKO_CSR && A->plan.kind == 1) && A->fmt != GKO_ELL && A->fmt != GKO_SELLP) return GKO_NOT_SUPPORTED;
+  if (sp.rel && (sp.solver != 1 || sp.rel->A64->fmt != A->fmt)) return GKO_NOT_SUPPORTED;
+  int dev = 0, coop = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return GKO_NOT_SUPPORTED;
+  }
+  if (!coop) return GKO_NOT_SUPPORTED;
+  switch (A->dtype) {
+    case GKO_F64:
+      return run<double, double>(A, b, static_cast<double*>(x), x_zero, sp, s, out);
+    case GKO_F32:
+      return run<float, float>(A, b, static_cast<float*>(x), x_zero, sp, s, out);
+    case GKO_BF16:
+      return run<float, __nv_bfloat16>(A, b, static_cast<float*>(x), x_zero, sp, s, out);
+  }
+  return GKO_NOT_SUPPORTED;
+}
+
+}  // namespace gko

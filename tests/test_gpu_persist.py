@@ -1,0 +1,111 @@
+"""The single-launch CG and BiCGSTAB at the edges of their launch shapes
+(blocks of 32-512 rows in one cluster, then one block per SM) against the
+oracle: both sides to 1e-12, solutions within 1e-8 (kappa * 1e-12 << 1e-8),
+the reported residual the true one, as tests/test_gpu_solvers.py."""
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_util import dev, host
+from paper_2006_14290_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def banded_system(n, half, spd, seed):
+    """Diagonally dominant band matrix: rows of 1 to 2*half+1 entries, ragged ends."""
+    rng = np.random.default_rng(seed)
+    offs = [k for k in range(-half, half + 1) if k == 0 or abs(k) in (1, half)]
+    cols = np.arange(n)[:, None] + np.array(offs)[None, :]
+    vals = rng.uniform(-1.0, -0.2, cols.shape)
+    if spd:
+        vals[:] = -1.0
+    vals[:, offs.index(0)] = len(offs) - 1 + 0.5
+    ok = (cols >= 0) & (cols < n)
+    rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+    return I.Csr(n, n, rp, cols[ok].astype(np.int32), vals[ok], f"band_{n}")
+
+
+def solve(G, name, M, b, tol=1e-12, maxit=3000, **opt):
+    xd = dev(np.zeros(b.size))
+    fn = G.gko_solve_cg if name == "cg" else G.gko_solve_bicgstab
+    res = fn(M, dev(b), xd, tol, maxit, G.opts(**opt) if opt else None)
+    return host(xd), res
+
+
+def check(G, name, A, M, seed=1, **opt):
+    b = np.random.default_rng(seed).uniform(-1, 1, A.n_rows)
+    x, res = solve(G, name, M, b, **opt)
+    xo, ro = O.solve(O.CG if name == "cg" else O.BICGSTAB, A, b, tol=1e-12, maxit=3000)
+    assert res.status == G.OK and ro.status == 0, res
+    assert np.linalg.norm(x - xo) <= 1e-8 * np.linalg.norm(xo)
+    true = np.linalg.norm(b - O.spmv_csr(A, x)) / np.linalg.norm(b)
+    assert true <= 1.01e-12 and abs(true - res.rel_residual) <= 1e-13
+    return b, x
+
+
+# block and cluster edges: 1 row, one warp, 16 blocks of 32/64/128/256/512 rows and one row more
+SIZES = [1, 2, 31, 32, 33, 512, 513, 1024, 1025, 2048, 2049, 4096, 4097, 8192, 8193, 9729, 19457, 38913, 77825]
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("name", ["cg", "bicgstab"])
+def test_shape_edges(gko, name, n):
+    G = gko
+    A = banded_system(n, 7, name == "cg", n)
+    b, x = check(G, name, A, G.from_csr(A))
+    x2, _ = solve(G, name, G.from_csr(A), b)
+    assert x.tobytes() == x2.tobytes()
+    check(G, name, A, G.from_csr(A), precision=G.PRECISION_MIXED_F32, preconditioner=G.PRECOND_JACOBI)
+
+
+@pytest.mark.parametrize("fmt", ["ell", "sellp32", "sellp128"])
+@pytest.mark.parametrize("n", [700, 9001, 100003])
+@pytest.mark.parametrize("name", ["cg", "bicgstab"])
+def test_padded_formats(gko, name, n, fmt):
+    """ELL and SELL-P (slices that end inside a block) against the same solve from CSR."""
+    G = gko
+    A = banded_system(n, 11, name == "cg", n)
+    M = G.from_csr(A)
+    M = G.gko_matrix_convert_to_ell(M) if fmt == "ell" else G.gko_matrix_convert_to_sellp(M, int(fmt[5:]))
+    check(G, name, A, M)
+    check(G, name, A, M, precision=G.PRECISION_MIXED_F32, refinement=G.REFINE_AUTO)
+
+
+@pytest.mark.parametrize("name", ["cg", "bicgstab"])
+def test_entries_that_do_not_fit_in_shared_memory(gko, name):
+    """Rows of about 400 entries: read from the matrix every iteration."""
+    G = gko
+    n, half = 20000, 200
+    rng = np.random.default_rng(4)
+    cols = np.arange(n)[:, None] + np.arange(-half, half + 1)[None, :]
+    vals = np.full(cols.shape, -1.0) if name == "cg" else rng.uniform(-1, 0, cols.shape)
+    vals[:, half] = 2 * half + 1.0
+    ok = (cols >= 0) & (cols < n)
+    rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+    A = I.Csr(n, n, rp, cols[ok].astype(np.int32), vals[ok], "wide")
+    check(G, name, A, G.from_csr(A))
+
+
+@pytest.mark.parametrize("n", [300, 20000])
+@pytest.mark.parametrize("name", ["cg", "bicgstab"])
+def test_scaled_and_special_right_hand_sides(gko, name, n):
+    """The sums keep their accuracy at any scale of b, zero stays zero, and
+    infinities and NaN end the solve as the reductions in FP64 do."""
+    G = gko
+    A = banded_system(n, 7, name == "cg", 3)
+    M = G.from_csr(A)
+    b = np.random.default_rng(2).uniform(-1, 1, n)
+    x1, r1 = solve(G, name, M, b)
+    for k in (-400, -100, 100, 400):  # powers of two: the same digits
+        xs, rs = solve(G, name, M, np.ldexp(b, k))
+        assert rs.status == G.OK and rs.iterations == r1.iterations and np.array_equal(xs, np.ldexp(x1, k))
+    xz, rz = solve(G, name, M, np.zeros(n))
+    assert rz.status == G.OK and rz.iterations == 0 and np.all(xz == 0) and rz.rel_residual == 0
+    bn = b.copy()
+    bn[n // 2] = np.nan
+    _, rn = solve(G, name, M, bn, maxit=5)
+    assert rn.status in (G.BREAKDOWN, G.NOT_CONVERGED) and np.isnan(rn.rel_residual)
+    bn[n // 2] = np.inf  # ||b|| is infinite: every finite residual meets rel_tol ||b||
+    _, ri = solve(G, name, M, bn, maxit=5)
+    assert np.isnan(ri.rel_residual)
