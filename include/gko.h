@@ -494,7 +494,10 @@ GKO_API int gko_batch_set_threshold(gko_batch B, int32_t warp_rows, void *stream
  * change is added to the FP64 x and r is replaced by b - A x computed in FP64
  * with the stored values; a system converges when that FP64 residual meets
  * rel_tol ||b_i||.  The FP32 values are made once (FP64 storage) or are the
- * stored ones (FP32 storage).  Bad arguments: GKO_INVALID_ARG.  Synchronises
+ * stored ones (FP32 storage).  Systems that fit on one SM (up to 4,096 rows,
+ * entries and p in 216 KB of shared memory) are solved there by blocks as wide
+ * as they need, whatever the schedule; the schedule serves the others and
+ * FP64 solves.  Bad arguments: GKO_INVALID_ARG.  Synchronises
  * `stream`. */
 GKO_API int gko_batch_set_precision(gko_batch B, int32_t precision, double reliable_delta, void *stream);
 

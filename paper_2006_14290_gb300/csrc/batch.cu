@@ -15,11 +15,13 @@
 #include <math.h>
 
 #include <algorithm>
+#include <iterator>
 #include <numeric>
 #include <type_traits>
 #include <vector>
 
 #include "common.cuh"
+#include "fx.cuh"
 #include "reduce.cuh"
 
 namespace gko {
@@ -528,6 +530,256 @@ __global__ void __launch_bounds__(THREADS) batch_cg_rel_kernel(BatchArgs a, int 
   }
 }
 
+// ------------------------------------------------ resident mixed solve --
+//
+// The mixed-precision solve (cg_group_rel's method) with everything an
+// iteration touches on the SM: the thread's R consecutive rows of r, p, q and
+// y in registers, p and the system's entries in shared memory.  Against
+// reading the entries from L2 every iteration and keeping the vectors in
+// shared memory this takes the L2 round trips out of each iteration; the dots
+// are sums of exact FP32 products in integers (fx_dot, warp_fx_sum), so the
+// FP64 pipe, which two FMAs per row and iteration kept half busy, does the
+// step scalars only.  What is left is bound by instruction issue, hence:
+// entries as {value, byte offset of the p they multiply} pairs in 16-byte
+// units of two rows (one load for two entries, no address arithmetic), padding
+// that points at a zero, and p stored by (row mod R, row / R), which keeps the
+// gathers of a stencil free of bank conflicts.
+// Blocks are as wide as the system needs (a launch per width, widest first,
+// on parallel branches), so that small systems share an SM.
+constexpr size_t kResSmemMax = 216 * 1024;
+
+// Shared memory of a block of `threads` threads with R rows each and K
+// entries a row: p with a zero after it, then the entries.
+__host__ __device__ constexpr size_t res_p_bytes(int rows) { return ((size_t)rows * 4 + 16 + 15) / 16 * 16; }
+__host__ __device__ constexpr size_t res_smem(int rows, int K) { return res_p_bytes(rows) + (size_t)rows * K * 8; }
+
+struct ResShared {
+  Fx part[2][32];
+  double out[4];
+  double rho, inv;  // r.r of the current residual, and its reciprocal
+};
+
+struct ResNothing {
+  __device__ void operator()() const {}
+};
+
+// Block sums of NV values: thread 0 runs fin(totals, out), the block reads
+// sh.out after the last barrier; meanwhile() is work of every thread that the
+// totals do not touch.
+template <int NV, typename F, typename W = ResNothing>
+__device__ __forceinline__ void res_step(const Fx (&f)[NV], ResShared& sh, F fin, W meanwhile = W{}) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  Fx s[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    s[k] = warp_fx_sum(f[k]);
+    if (lane == 0) sh.part[k][w] = s[k];
+  }
+  __syncthreads();
+  if (w == 0) {
+    double t[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      if (nw > 1) s[k] = warp_fx_sum(lane < nw ? sh.part[k][lane] : Fx{0, 1});
+      t[k] = fx_double(s[k]);
+    }
+    if (lane == 0) fin(t, sh.out);
+  }
+  meanwhile();
+  __syncthreads();
+}
+
+template <int R, typename VT>
+__global__ void __launch_bounds__(512, R == 8 ? 1 : 2) batch_res_kernel(BatchArgs a, const int32_t* __restrict__ systems) {
+  extern __shared__ __align__(16) unsigned char res_mem[];
+  __shared__ ResShared sh;
+  const int NT = blockDim.x, RB = NT * R, tid = threadIdx.x;
+  const int sys = systems[blockIdx.x];
+  const int64_t r0 = a.row_off[sys], k0 = a.ell_off[sys];
+  const int n = (int)(a.row_off[sys + 1] - r0), K = a.ell_k[sys];
+  const int32_t* ecol = a.ell_col + k0;
+  const VT* eval = static_cast<const VT*>(a.ell_val) + k0;
+  const float* eval32 = a.ell_val32 + k0;
+  const double* b = a.b + r0;
+  double* x = a.x + r0;
+  const int i0 = tid * R;  // the thread's rows i0 .. i0 + R - 1
+  float* sp = reinterpret_cast<float*>(res_mem);  // row i at (i % R) NT + i / R; sp[RB] = 0
+  float4* se = reinterpret_cast<float4*>(res_mem + res_p_bytes(RB)) + tid;  // [k][row pair][thread]
+  for (int k = 0; k < K; ++k)
+#pragma unroll
+    for (int j = 0; j < R; j += 2) {
+      float v[2] = {0.0f, 0.0f};
+      int off[2] = {4 * RB, 4 * RB};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = i0 + j + u;
+        const int32_t c = i < n ? ecol[(int64_t)k * n + i] : -1;
+        if (c >= 0) {
+          v[u] = eval32[(int64_t)k * n + i];
+          off[u] = 4 * ((c % R) * NT + c / R);
+        }
+      }
+      se[(size_t)(k * (R / 2) + j / 2) * NT] = make_float4(v[0], __int_as_float(off[0]), v[1], __int_as_float(off[1]));
+    }
+  if (tid == 0) sp[RB] = 0.0f;
+  float r[R], p[R], y[R], q[R];
+  // A x of the thread's rows with the stored values and the FP64 x
+  auto row64 = [&](int i) -> double {
+    double s = 0.0;
+    for (int k = 0; k < K; ++k) {
+      const int64_t o = (int64_t)k * n + i;
+      const int32_t c = ecol[o];
+      if (c >= 0) s = __fma_rn(ldv(eval, o), x[c], s);
+    }
+    return s;
+  };
+  // r = fl32(b - A x); sums ||b - A x||^2 and r.r
+  auto replace = [&](Fx (&f)[2]) {
+    double tt = 0.0;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int i = i0 + j;
+      r[j] = 0.0f;
+      if (i >= n) continue;
+      const double ti = b[i] - row64(i);
+      r[j] = __double2float_rn(ti);
+      tt = __fma_rn(ti, ti, tt);
+    }
+    f[0] = fx_of(tt);
+    f[1] = fx_dot(r, r);
+  };
+  double bb = 0.0;
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int i = i0 + j;
+    if (i < n) bb = __fma_rn(b[i], b[i], bb);
+  }
+  Fx f1[1] = {fx_of(bb)}, f2[2];
+  replace(f2);
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    p[j] = r[j];
+    y[j] = 0.0f;
+    sp[j * NT + tid] = p[j];
+  }
+  // the step scalars live in thread 0
+  double nb = 0.0, tol = 0.0, tol2 = 0.0, maxrr2 = 0.0, res = 0.0;
+  const double delta2 = a.delta * a.delta;
+  res_step<1>(f1, sh, [&](const double (&t)[1], double*) { nb = sqrt(t[0]); });
+  res_step<2>(f2, sh, [&](const double (&t)[2], double* o) {
+    tol = a.rel_tol * nb;
+    tol2 = tol * tol;
+    maxrr2 = t[0];
+    sh.rho = t[1];
+    const double tn = sqrt(t[0]);
+    res = nb > 0.0 ? tn / nb : 0.0;
+    o[0] = nb == 0.0 ? 2.0 : tn <= tol ? 1.0 : 0.0;
+  });
+  int status = kBRun, it = 0, updates = 0;
+  if (flag_on(sh.out[0])) {
+    status = kBOk;
+    if (sh.out[0] == 2.0)
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        if (i0 + j < n) x[i0 + j] = 0.0;
+  }
+  const bool helper = NT > 32 ? tid == 32 : false;  // forms 1 / rho while the block multiplies
+  auto fold = [&] {  // x += y, y = 0
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int i = i0 + j;
+      if (i < n) x[i] += widen(y[j]);
+      y[j] = 0.0f;
+    }
+    __syncthreads();
+  };
+  while (status == kBRun && it < a.maxit) {
+    if (helper) sh.inv = 1.0 / sh.rho;
+#pragma unroll
+    for (int j = 0; j < R; ++j) q[j] = 0.0f;
+    const float4* ek = se;
+#pragma unroll 5
+    for (int k = 0; k < K; ++k, ek += (R / 2) * NT)
+#pragma unroll
+      for (int j = 0; j < R; j += 2) {
+        const float4 e = ek[(j / 2) * NT];
+        q[j] = __fmaf_rn(e.x, *reinterpret_cast<const float*>(res_mem + __float_as_int(e.y)), q[j]);
+        q[j + 1] = __fmaf_rn(e.z, *reinterpret_cast<const float*>(res_mem + __float_as_int(e.w)), q[j + 1]);
+      }
+    f1[0] = fx_dot(p, q);
+    res_step<1>(f1, sh, [&](const double (&t)[1], double* o) {
+      const bool up = t[0] > 0.0;
+      o[0] = up ? 1.0 : 0.0;
+      o[1] = lin_of(up ? fast_div(sh.rho, t[0]) : 0.0).pack();
+    });
+    if (!flag_on(sh.out[0])) {
+      status = kBBreak;
+      break;
+    }
+    const Lin<float> ay = Lin<float>::unpack(sh.out[1]), ar(-ay.hi, -ay.lo);
+#pragma unroll
+    for (int j = 0; j < R; ++j) r[j] = ar(q[j], r[j]);
+    f1[0] = fx_dot(r, r);
+    res_step<1>(f1, sh, [&](const double (&t)[1], double* o) {
+      const double rr = t[0], rho = sh.rho;
+      maxrr2 = rr > maxrr2 ? rr : maxrr2;
+      o[0] = (rr <= tol2 || rr < delta2 * maxrr2) ? 1.0 : 0.0;
+      double beta;
+      if (NT > 32) {
+        // rr / rho from the helper's reciprocal, its error removed with the exact residual
+        const double inv = sh.inv, g = rr * inv, e = __fma_rn(-rho, g, rr);
+        beta = isfinite(e) ? __fma_rn(e, inv, g) : rr / rho;
+      } else {
+        beta = fast_div(rr, rho);
+      }
+      o[1] = lin_of(beta).pack();
+      o[2] = rho;  // before this step
+      sh.rho = rr;
+    }, [&] {  // while warp 0 derives beta
+#pragma unroll
+      for (int j = 0; j < R; ++j) y[j] = ay(p[j], y[j]);
+    });
+    ++it;
+    Lin<float> bp = Lin<float>::unpack(sh.out[1]);
+    if (flag_on(sh.out[0])) {  // reliable update
+      const double rho_old = sh.out[2];
+      fold();
+      replace(f2);
+      ++updates;
+      res_step<2>(f2, sh, [&](const double (&t)[2], double* o) {
+        res = sqrt(t[0]) / nb;
+        o[0] = t[0] <= tol2 ? 1.0 : 0.0;
+        maxrr2 = t[0];
+        sh.rho = t[1];
+        o[1] = Lin<float>(t[1] / rho_old).pack();
+      });
+      if (flag_on(sh.out[0])) {
+        status = kBOk;
+        break;
+      }
+      bp = Lin<float>::unpack(sh.out[1]);
+    }
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      p[j] = bp(p[j], r[j]);
+      sp[j * NT + tid] = p[j];
+    }
+    __syncthreads();
+  }
+  if (status == kBRun) status = kBNotConv;
+  if (status != kBOk) {  // fold what moved since the last update; report the true residual
+    fold();
+    replace(f2);
+    res_step<2>(f2, sh, [&](const double (&t)[2], double*) { res = nb > 0.0 ? sqrt(t[0]) / nb : 0.0; });
+  }
+  if (tid == 0) {
+    a.iters[sys] = it;
+    a.relres[sys] = res;
+    a.status[sys] = status;
+    a.updates[sys] = updates;
+  }
+}
+
 // Persistent batched CG: blocks of THREADS threads take work items from an
 // atomic queue, largest systems first; a block item is one system solved by
 // the whole block, a warp item THREADS/32 systems, one per warp.
@@ -591,6 +843,18 @@ struct gko_batch_s {
   int32_t ell = 0;               // 1: solve from the ELL arrays
   int n_items = 0;
   int block_rows = 0;
+  // mixed precision: the systems solved resident on an SM, in launches of one
+  // block width each (widest first), and the work items of the others
+  struct ResClass {
+    int threads, rows, first, count, slots;  // rows per thread; slots: longest row
+  };
+  std::vector<ResClass> res_classes;
+  std::vector<char> resident;  // per system
+  Buf res_systems, rest_items;
+  int n_rest = 0, rest_rows = 0;
+  // the branches of their launch
+  std::vector<cudaStream_t> branches;
+  std::vector<cudaEvent_t> events;
   // cached graph of (queue reset + kernel)
   cudaGraphExec_t exec = nullptr;
   const double* g_b = nullptr;
@@ -600,35 +864,50 @@ struct gko_batch_s {
   cudaStream_t g_stream = nullptr;
   ~gko_batch_s() {
     if (exec) cudaGraphExecDestroy(exec);
+    for (cudaEvent_t e : events) cudaEventDestroy(e);
+    for (cudaStream_t s : branches) cudaStreamDestroy(s);
   }
 };
 
 namespace gko {
 
-static int build_items(gko_batch B, int32_t threshold, cudaStream_t s) {
-  threshold = std::min(threshold, kWarpMaxRows);
+// Work items of the systems `order` lists, largest first: a block item each
+// above the threshold, then warp items.
+static int make_items(const gko_batch_s* B, const std::vector<int32_t>& at, int32_t threshold, Buf* out, int* n_items,
+                      int* block_rows, cudaStream_t s) {
   std::vector<int2> items;
-  int block_rows = 0;
+  *block_rows = 0;
   size_t i = 0;
-  const size_t n = B->h_order.size();
-  while (i < n && B->h_rows[B->h_order[i]] > threshold) {
-    block_rows = std::max<int>(block_rows, (int)B->h_rows[B->h_order[i]]);
-    items.push_back(make_int2((int)(i << 1) | 0, 1));
+  const size_t n = at.size();
+  while (i < n && B->h_rows[B->h_order[at[i]]] > threshold) {
+    *block_rows = std::max<int>(*block_rows, (int)B->h_rows[B->h_order[at[i]]]);
+    items.push_back(make_int2((int)(at[i] << 1) | 0, 1));
     ++i;
   }
   const size_t per_item = (size_t)B->threads / kWarp;
-  while (i < n) {
-    const int cnt = (int)std::min<size_t>(per_item, n - i);
-    items.push_back(make_int2((int)(i << 1) | 1, cnt));
+  while (i < n) {  // consecutive positions of the order only: an item is a first position and a count
+    size_t cnt = 1;
+    while (cnt < per_item && i + cnt < n && at[i + cnt] == at[i] + (int32_t)cnt) ++cnt;
+    items.push_back(make_int2((int)(at[i] << 1) | 1, (int)cnt));
     i += cnt;
   }
-  GKO_TRY(alloc(sizeof(int2) * std::max<size_t>(1, items.size()), &B->items));
+  GKO_TRY(alloc(sizeof(int2) * std::max<size_t>(1, items.size()), out));
   if (!items.empty())
-    GKO_TRY_CUDA(cudaMemcpyAsync(B->items->ptr, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice, s));
+    GKO_TRY_CUDA(cudaMemcpyAsync((*out)->ptr, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice, s));
   GKO_TRY_CUDA(cudaStreamSynchronize(s));
+  *n_items = (int)items.size();
+  return GKO_OK;
+}
+
+static int build_items(gko_batch B, int32_t threshold, cudaStream_t s) {
+  threshold = std::min(threshold, kWarpMaxRows);
+  std::vector<int32_t> all(B->h_order.size()), rest;
+  std::iota(all.begin(), all.end(), 0);
+  for (int32_t i : all)
+    if (!B->resident[B->h_order[i]]) rest.push_back(i);
+  GKO_TRY(make_items(B, all, threshold, &B->items, &B->n_items, &B->block_rows, s));
+  GKO_TRY(make_items(B, rest, threshold, &B->rest_items, &B->n_rest, &B->rest_rows, s));
   B->threshold = threshold;
-  B->n_items = (int)items.size();
-  B->block_rows = block_rows;
   if (B->exec) {
     cudaGraphExecDestroy(B->exec);
     B->exec = nullptr;
@@ -636,12 +915,83 @@ static int build_items(gko_batch B, int32_t threshold, cudaStream_t s) {
   return GKO_OK;
 }
 
+// The resident mixed solve's classes.  8 rows a thread (128 registers) repeat
+// the per-warp work of the sums less often (89 instructions per row and
+// iteration against 114 with 4 rows and 64 registers), but leave an SM only 16
+// warps: 8 rows from 1,025 rows on, where one or two blocks fill the shared
+// memory anyway (600 systems of 2,116-4,096 rows: 9.7 ms, with 4 rows 10.1),
+// 4 rows below (4,096 systems of 64-256 rows: 1.84 ms with 8, 1.45 with 4),
+// one warp with 2 for the smallest.
+constexpr struct {
+  int threads, rows;
+} kResWidths[] = {{512, 8}, {448, 8}, {384, 8}, {320, 8}, {256, 8}, {224, 8}, {192, 8}, {160, 8}, {256, 4},
+                  {224, 4}, {192, 4}, {160, 4}, {128, 4}, {96, 4},  {64, 4},  {32, 4},  {32, 2}};
+
+static int build_resident(gko_batch B, const std::vector<int32_t>& slots, cudaStream_t s) {
+  B->resident.assign(B->h_rows.size(), 0);
+  std::vector<int32_t> systems;
+  for (size_t w = 0; w < std::size(kResWidths); ++w) {
+    const int64_t most = (int64_t)kResWidths[w].threads * kResWidths[w].rows;
+    const int64_t least = w + 1 < std::size(kResWidths) ? (int64_t)kResWidths[w + 1].threads * kResWidths[w + 1].rows : 0;
+    gko_batch_s::ResClass c{kResWidths[w].threads, kResWidths[w].rows, (int)systems.size(), 0, 0};
+    for (int32_t sys : B->h_order) {
+      const int64_t n = B->h_rows[sys];
+      if (n > most || n <= least || res_smem((int)most, slots[sys]) > kResSmemMax) continue;
+      systems.push_back(sys);
+      B->resident[sys] = 1;
+      c.slots = std::max(c.slots, slots[sys]);
+      ++c.count;
+    }
+    if (c.count) B->res_classes.push_back(c);
+  }
+  GKO_TRY(alloc(sizeof(int32_t) * std::max<size_t>(1, systems.size()), &B->res_systems));
+  if (!systems.empty())
+    GKO_TRY_CUDA(cudaMemcpyAsync(B->res_systems->ptr, systems.data(), sizeof(int32_t) * systems.size(),
+                                 cudaMemcpyHostToDevice, s));
+  GKO_TRY_CUDA(cudaStreamSynchronize(s));
+  return GKO_OK;
+}
+
 static size_t batch_smem(const gko_batch_s* B) {
   // FP64: r, p, q as doubles; mixed: r, p, q, y as floats
   const size_t per = B->mixed ? 4 * sizeof(float) : 3 * sizeof(double);
-  const size_t blk = per * B->block_rows;
+  const size_t blk = per * (B->mixed ? B->rest_rows : B->block_rows);
   const size_t wrp = B->threshold > 0 ? (size_t)(B->threads / kWarp) * per * kWarpMaxRows : 0;
   return std::max<size_t>(std::max(blk, wrp), 16);
+}
+
+// The resident classes of a mixed solve on parallel branches forked from s
+// and joined to it again (captured into the batch's graph).
+template <typename VT>
+static int resident_launch(gko_batch B, const BatchArgs& a, cudaStream_t s) {
+  for (auto kern : {batch_res_kernel<2, VT>, batch_res_kernel<4, VT>, batch_res_kernel<8, VT>})
+    GKO_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax));
+  const size_t branches = B->res_classes.size();
+  while (B->branches.size() + 1 < branches) {
+    cudaStream_t h;
+    GKO_TRY_CUDA(cudaStreamCreateWithFlags(&h, cudaStreamNonBlocking));
+    B->branches.push_back(h);
+  }
+  while (B->events.size() < branches) {
+    cudaEvent_t e;
+    GKO_TRY_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    B->events.push_back(e);
+  }
+  if (branches > 1) GKO_TRY_CUDA(cudaEventRecord(B->events[0], s));
+  for (size_t i = 0; i < branches; ++i) {
+    const auto& c = B->res_classes[i];
+    cudaStream_t h = i ? B->branches[i - 1] : s;
+    if (i) GKO_TRY_CUDA(cudaStreamWaitEvent(h, B->events[0], 0));
+    auto kern = c.rows == 2 ? batch_res_kernel<2, VT> : c.rows == 4 ? batch_res_kernel<4, VT> : batch_res_kernel<8, VT>;
+    const size_t smem = res_smem(c.threads * c.rows, c.slots);
+    kern<<<(unsigned)c.count, (unsigned)c.threads, smem, h>>>(a, ptr<int32_t>(B->res_systems) + c.first);
+    GKO_TRY_CUDA(cudaGetLastError());
+    if (i) {
+      GKO_TRY_CUDA(cudaEventRecord(B->events[i], h));
+    }
+  }
+  for (size_t i = 1; i < branches; ++i) GKO_TRY_CUDA(cudaStreamWaitEvent(s, B->events[i], 0));
+  return GKO_OK;
 }
 
 template <int T, typename VT, bool E>
@@ -686,10 +1036,16 @@ static int batch_launch(gko_batch B, const double* b, double* x, double tol, int
   GKO_TRY_CUDA(cudaMemsetAsync(B->queue->ptr, 0, sizeof(unsigned), s));
   if (!B->mixed) GKO_TRY_CUDA(cudaMemsetAsync(B->updates->ptr, 0, sizeof(int32_t) * B->count, s));
   const bool f64 = B->dtype == GKO_F64;
+  if (B->mixed) {
+    GKO_TRY(f64 ? resident_launch<double>(B, a, s) : resident_launch<float>(B, a, s));
+    if (B->n_rest == 0) return GKO_OK;
+    a.items = ptr<int2>(B->rest_items);
+    a.n_items = B->n_rest;
+  }
   switch (B->threads * 4 + (f64 ? 2 : 0) + (B->ell ? 1 : 0)) {
 #define GKO_BATCH_CASE(T, VT, E) \
   case T * 4 + (std::is_same<VT, double>::value ? 2 : 0) + (E ? 1 : 0): \
-    return batch_launch_t<T, VT, E>(a, B->n_items, B->block_rows, smem, B->mixed != 0, s);
+    return batch_launch_t<T, VT, E>(a, a.n_items, B->mixed ? B->rest_rows : B->block_rows, smem, B->mixed != 0, s);
 #define GKO_BATCH_T(T) \
   GKO_BATCH_CASE(T, double, false) GKO_BATCH_CASE(T, double, true) GKO_BATCH_CASE(T, float, false) \
   GKO_BATCH_CASE(T, float, true)
@@ -790,7 +1146,7 @@ static int build_ell(gko_batch B, const int64_t* row_off, const int64_t* nnz_off
   }
   GKO_TRY_CUDA(cudaStreamSynchronize(s));  // the host arrays above go out of scope
   B->ell_slots = slots;
-  return GKO_OK;
+  return build_resident(B, kk, s);
 }
 
 }  // namespace gko

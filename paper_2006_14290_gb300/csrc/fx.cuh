@@ -92,4 +92,73 @@ __device__ __forceinline__ double fx_double(const Fx& f) {
                : d * __hiloint2double(2046 << 20, 0) * __hiloint2double((k - 1023 + 1023) << 20, 0);
 }
 
+// Sum of N <= 8 products a[i] * b[i] of FP32 numbers, exact like the FP64
+// products would be (24 x 24 = 48 bits), added on the scale of the largest:
+// about 25 integer instructions a product instead of two widenings and an
+// FP64 FMA, whose 16 cycles of the SM's one FP64 pipe are its cost.  FP32
+// subnormals count as zero (as in widen); infinities and NaN go through FP64.
+template <int N>
+__device__ __forceinline__ Fx fx_dot(const float (&a)[N], const float (&b)[N]) {
+  static_assert(N <= 8, "eight 60-bit products");
+  long long x[N];
+  unsigned e[N], E = 1u << 23, top = 0u;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const unsigned ua = __float_as_uint(a[i]), ub = __float_as_uint(b[i]);
+    const unsigned fa = ua & 0x7f800000u, fb = ub & 0x7f800000u;
+    top = max(top, max(fa, fb));
+    const bool zero = min(fa, fb) == 0u;
+    const int s = (int)(ua ^ ub) >> 31;
+    int ma = (int)(((ua << 5) & 0x0fffffe0u) | 0x10000000u);  // 24 bits, up by 5
+    ma = zero ? 0 : (ma ^ s) - s;
+    x[i] = (long long)ma * (int)(((ub << 7) & 0x3fffff80u) | 0x40000000u);  // 24 bits, up by 7
+    e[i] = zero ? 0u : fa + fb;
+    E = max(E, e[i]);
+  }
+  if (top == 0x7f800000u) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) s = __fma_rn(widen(a[i]), widen(b[i]), s);
+    return fx_of(s);
+  }
+  long long s = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) s += x[i] >> min((E - e[i]) >> 23, 63u);
+  // m 2^(e - 300) = (m 2^12) 2^(e - 312)
+  return Fx{s, (int)(E >> 23) - 312 + kFxBias};
+}
+
+// a / b, b != 0: reciprocal estimate, one Newton-Raphson step (40 correct
+// bits), quotient and one correction of it with its exact residual (Markstein,
+// IBM J. Res. Dev. 34, 1990), which leaves about the rounding error of the
+// quotient: 5 dependent FP64 operations of 67 cycles instead of 552 cycles of
+// IEEE division, on the critical path of every iteration.  Operands whose
+// estimate or residual could leave the normal range divide as usual.
+__device__ __forceinline__ double fast_div(double a, double b) {
+  const unsigned eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu, ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
+  if (eb - 523u > 1000u || ea - 523u > 1000u) return a / b;  // exponents outside 2^-500 .. 2^500
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+  r = __fma_rn(r, __fma_rn(-b, r, 1.0), r);
+  const double q = a * r;
+  return __fma_rn(r, __fma_rn(-b, q, a), q);
+}
+
+// The float pair of an FP64 scalar (Lin<float>: hi = a rounded to FP32, lo =
+// what is left, rounded) in integer operations: about 110 cycles on the
+// critical path of a step instead of 365 for the conversions and the FP64
+// subtraction.  Scalars outside 2^-60 .. 2^120 convert as usual.
+__device__ __forceinline__ Lin<float> lin_of(double a) {
+  const unsigned h = (unsigned)__double2hiint(a);
+  const unsigned e = (h >> 20) & 0x7ffu;
+  if (e - 963u > 180u) return Lin<float>(a);
+  const long long m = (long long)(((unsigned long long)__double_as_longlong(a) & 0xfffffffffffffull) | (1ull << 52));
+  const unsigned top = (unsigned)((m + (1ll << 28)) >> 29);  // 24 bits, or 2^24
+  const int rest = (int)(m - ((long long)top << 29));
+  const unsigned sign = h & 0x80000000u;
+  const float lo = __int2float_rn(rest);  // times 2^(e - 1075)
+  const unsigned lb = rest ? __float_as_uint(lo) + ((e - 1075u) << 23) : 0u;
+  return Lin<float>(__uint_as_float(sign | (((e - 896u) << 23) + (top - (1u << 23)))), __uint_as_float(lb ^ sign));
+}
+
 }  // namespace gko

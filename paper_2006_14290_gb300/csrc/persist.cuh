@@ -269,7 +269,7 @@ __device__ __forceinline__ bool pk_step(const double* v, PkShared<NT, MODE>& sh,
 template <typename T>
 __device__ __forceinline__ double pk_pack(double a) {
   if constexpr (sizeof(T) == 8) return a;
-  else return Lin<float>(a).pack();
+  else return lin_of(a).pack();
 }
 template <typename T>
 __device__ __forceinline__ Lin<T> pk_lin(double p) {
@@ -277,22 +277,6 @@ __device__ __forceinline__ Lin<T> pk_lin(double p) {
   else return Lin<float>::unpack(p);
 }
 __device__ __forceinline__ bool pk_flag(double f) { return __double_as_longlong(f) != 0; }
-
-// a / b, b != 0: reciprocal estimate, one Newton-Raphson step (40 correct
-// bits), quotient and one correction of it with its exact residual (Markstein,
-// IBM J. Res. Dev. 34, 1990), which leaves about the rounding error of the
-// quotient: 5 dependent FP64 operations of 67 cycles instead of 552 cycles of
-// IEEE division, on the critical path of every iteration.  Operands whose
-// estimate or residual could leave the normal range divide as usual.
-__device__ __forceinline__ double pk_div(double a, double b) {
-  const unsigned eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu, ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
-  if (eb - 523u > 1000u || ea - 523u > 1000u) return a / b;  // exponents outside 2^-500 .. 2^500
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
-  r = __fma_rn(r, __fma_rn(-b, r, 1.0), r);
-  const double q = a * r;
-  return __fma_rn(r, __fma_rn(-b, q, a), q);
-}
 
 // sqrt(rr) <= tol, without the square root where rr is clearly above tol^2
 // (tol2 = tol * tol; the margin covers the rounding of both)
@@ -574,7 +558,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
     for (int j = 0; j < RPT; ++j) v1[0] += wd(pj[j]) * wd(qj[j]);
     if (!pk_step<NT, MODE, kPubNone, 1>(v1, sh, a.slots, a.err, seq, [&](const double (&t)[1], double* o) {
           const bool up = t[0] > 0.0;
-          const double alpha = up ? pk_div(rho, t[0]) : 0.0;
+          const double alpha = up ? fast_div(rho, t[0]) : 0.0;
           o[0] = up ? 1.0 : 0.0;
           o[1] = pk_pack<T>(alpha);
           o[2] = pk_pack<T>(-alpha);
@@ -862,7 +846,7 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
     if (!pk_step<NT, MODE, FLY ? kPubVec : kPubNone, 1>(v1, sh, a.slots, a.err, seq, [&](const double (&t)[1], double* o) {
           const bool up = t[0] != 0.0;
           o[0] = up ? 1.0 : 0.0;
-          if (up) alpha = pk_div(rho_new, t[0]);
+          if (up) alpha = fast_div(rho_new, t[0]);
           o[1] = pk_pack<T>(alpha);
           o[2] = pk_pack<T>(-alpha);
         })) {
@@ -912,7 +896,7 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
           const bool half = pk_meets(t[2], tol, tol2);
           o[0] = half ? 1.0 : 0.0;
           o[1] = t[1] == 0.0 ? 1.0 : 0.0;
-          if (!half && t[1] != 0.0) omega = pk_div(t[0], t[1]);
+          if (!half && t[1] != 0.0) omega = fast_div(t[0], t[1]);
           o[2] = pk_pack<T>(omega);
           o[3] = pk_pack<T>(-omega);
         })) {

@@ -109,3 +109,39 @@ def test_scaled_and_special_right_hand_sides(gko, name, n):
     bn[n // 2] = np.inf  # ||b|| is infinite: every finite residual meets rel_tol ||b||
     _, ri = solve(G, name, M, bn, maxit=5)
     assert np.isnan(ri.rel_residual)
+
+
+def test_batch_mixed_widths_and_long_rows(gko):
+    """The batched mixed solve at the edges of its block widths, and next to
+    systems whose rows are too long for it (the queued kernels take those):
+    per system the oracle's solution within 1e-8, the true residual reported."""
+    G = gko
+    rng = np.random.default_rng(6)
+    sizes = [1, 3, 63, 64, 65, 128, 129, 255, 256, 257, 1023, 1024, 1025, 1281, 2049, 4095, 4096, 4097, 5000]
+    systems = [banded_system(n, 7, True, n) for n in sizes]
+    for n in (40, 300, 1500):  # 61 entries a row
+        half = 30
+        cols = np.arange(n)[:, None] + np.arange(-half, half + 1)[None, :]
+        vals = np.full(cols.shape, -1.0)
+        vals[:, half] = 2 * half + 0.5
+        ok = (cols >= 0) & (cols < n)
+        rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+        systems.append(I.Csr(n, n, rp, cols[ok].astype(np.int32), vals[ok], "long"))
+    bs = [rng.uniform(-1, 1, A.n_rows) for A in systems]
+    bs[4][:] = 0.0
+    bs[7] = np.ldexp(bs[7], -60)
+    B = G.Batch(systems)
+    B.set_precision(G.PRECISION_MIXED_F32)
+    xd = dev(np.zeros(B.total_rows))
+    code, it, rr, st = B.cg(dev(np.concatenate(bs)), xd, 1e-12, 5000)
+    assert code == G.OK and np.all(st == G.OK)
+    x = host(xd)
+    for i, A in enumerate(systems):
+        xi = x[B.row_off[i]:B.row_off[i + 1]]
+        if i == 4:
+            assert it[i] == 0 and np.all(xi == 0) and rr[i] == 0
+            continue
+        xo, ro = O.cg(A, bs[i], tol=1e-12, maxit=5000)
+        assert ro.status == 0 and np.linalg.norm(xi - xo) <= 1e-8 * np.linalg.norm(xo), i
+        true = np.linalg.norm(bs[i] - O.spmv_csr(A, xi)) / np.linalg.norm(bs[i])
+        assert true <= 1.01e-12 and abs(true - rr[i]) <= 1e-14
