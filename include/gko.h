@@ -244,7 +244,8 @@ GKO_API int gko_spmv_host(const double *alpha, gko_matrix A, const void *x_host,
  * allocate device memory at the time they multiply (their memory is owned by
  * another allocator, or an allocation's possible implicit synchronisation is
  * not acceptable in their loop).  It always runs the tiled segmented-reduction
- * kernels, whatever plan the handle carries, so its y equals gko_spmv's
+ * kernels (the same ones gko_spmv takes by default, with or without carries
+ * as the matrix asks), whatever plan the handle carries, so its y equals gko_spmv's
  * within the SpMV tolerance (bit-identical under the default plan; a handle
  * set to the row-block COO plan sums in another order).  The per-tile
  * carries live in a fixed 2 MiB device array inside the library instead of

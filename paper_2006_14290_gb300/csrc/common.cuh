@@ -117,6 +117,13 @@ struct CsrPlan {
   int64_t merge_tiles = 0;
   Buf seg_row;         // int32[tiles+1]    nonzero split: row of the first nonzero of each tile
   int64_t seg_tiles = 0;
+  // nonzero split and COO in row-aligned tiles: tile t holds the rows that
+  // start at nonzeros [t W, (t+1) W).
+  // CSR: seg_row with tiles of W; COO: tile_start
+  Buf tile_start;       // COO: int32[tiles+1]  first entry of each tile, behind the row indices
+  int64_t tile_start_at = 0;  // ... at this int32 offset
+  int64_t tiles = 0;    // 0: the kernels with carries
+  int32_t tile_width = 0;  // W
   // COO handles: kind 1 runs the row-block kernel over the COO arrays, any
   // other kind the tiled segmented reduction.
   Buf coo_rb;          // int32[n_rb+1]     first COO entry of each row block of (128/S)*R rows

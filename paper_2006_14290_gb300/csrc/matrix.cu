@@ -316,14 +316,62 @@ __global__ void seg_rows_kernel(int64_t n, int64_t tiles, int64_t tile, const in
   }
 }
 
+// First entry of each row-aligned tile: the first row start at or behind
+// nonzero t * width (0 for tile 0, the end for t = tiles).
+__global__ void tile_starts_kernel(int64_t n, int64_t tiles, int64_t width, const int32_t* __restrict__ rp,
+                                   int32_t* __restrict__ out) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t <= tiles; t += (int64_t)gridDim.x * blockDim.x) {
+    int64_t lo = 0, hi = n;
+    if (t == tiles) lo = n;
+    else if (t > 0)
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if ((int64_t)rp[mid] < t * width) lo = mid + 1;
+        else hi = mid;
+      }
+    out[t] = rp[lo];
+  }
+}
+
+// Row-aligned tiles of a matrix (0: the kernels with carries, see spmv.cuh).
+static int64_t tile_count(int64_t n, int64_t nnz, int32_t max_len) {
+  if (nnz == 0 || max_len > kTileRowMax || (nnz > kTileNnzMax && nnz < kTileRowMean * n)) return 0;
+  const int64_t w = tile_width_for(max_len);
+  return (nnz + w - 1) / w;
+}
+
+// Tile starts of a COO part whose rows' entries rp delimits, written behind
+// its row indices (coo_row holds `nnz` of them, then tiles + 1 starts).
+static int build_tile_starts(gko_matrix m, const int32_t* rp, int64_t nnz, int32_t max_len, cudaStream_t s) {
+  CsrPlan& p = m->plan;
+  p.tiles = tile_count(m->n_rows, nnz, max_len);
+  if (!p.tiles) return GKO_OK;
+  p.tile_start = m->coo_row;
+  p.tile_width = tile_width_for(max_len);
+  p.tile_start_at = (nnz + 3) / 4 * 4;
+  tile_starts_kernel<<<grid_for(p.tiles + 1), 256, 0, s>>>(m->n_rows, p.tiles, p.tile_width, rp,
+                                                           ptr<int32_t>(m->coo_row) + p.tile_start_at);
+  GKO_TRY_CUDA(cudaGetLastError());
+  return GKO_OK;
+}
+
+// int32 words of a COO part's row indices and the tile starts behind them
+static int64_t coo_row_words(int64_t n, int64_t nnz, int32_t max_len) {
+  const int64_t t = tile_count(n, nnz, max_len);
+  return t ? (nnz + 3) / 4 * 4 + t + 1 : nnz;
+}
+
 static int build_seg_rows(gko_matrix m, cudaStream_t s) {
   CsrPlan& p = m->plan;
   p.seg_row.reset();
   p.seg_tiles = 0;
+  p.tiles = 0;
   if (p.kind != 3 || m->nnz == 0) return GKO_OK;
-  const int64_t tiles = (m->nnz + kCooTile - 1) / kCooTile;
+  p.tiles = tile_count(m->n_rows, m->nnz, p.max_len);
+  p.tile_width = p.tiles ? tile_width_for(p.max_len) : kCooTile;
+  const int64_t tiles = p.tiles ? p.tiles : (m->nnz + kCooTile - 1) / kCooTile;
   GKO_TRY(alloc(sizeof(int32_t) * (tiles + 1), &p.seg_row));
-  seg_rows_kernel<<<grid_for(tiles + 1), 256, 0, s>>>(m->n_rows, tiles, kCooTile, ptr<int32_t>(m->row_ptr),
+  seg_rows_kernel<<<grid_for(tiles + 1), 256, 0, s>>>(m->n_rows, tiles, p.tile_width, ptr<int32_t>(m->row_ptr),
                                                       ptr<int32_t>(p.seg_row));
   GKO_TRY_CUDA(cudaGetLastError());
   GKO_TRY_CUDA(cudaStreamSynchronize(s));
@@ -638,6 +686,8 @@ int gko_matrix_set_plan(gko_matrix m, int32_t kernel, int32_t S, int32_t R, int3
       q.merge_tiles = m->plan.merge_tiles;
       q.seg_row = m->plan.seg_row;
       q.seg_tiles = m->plan.seg_tiles;
+      q.tiles = m->plan.tiles;
+      q.tile_width = m->plan.tile_width;
     }
   }
   return GKO_OK;
@@ -743,9 +793,10 @@ int gko_matrix_convert_to_coo(gko_matrix csr, void* stream, gko_matrix* out) {
   m->plan.S = csr->plan.S;
   m->plan.R = csr->plan.R;
   m->plan.cap = std::min<int32_t>(csr->plan.cap, kCooRbMaxCap);
-  GKO_TRY(alloc(sizeof(int32_t) * nnz, &m->coo_row));
+  GKO_TRY(alloc(sizeof(int32_t) * coo_row_words(csr->n_rows, nnz, csr->plan.max_len), &m->coo_row));
   GKO_TRY(alloc(sizeof(int32_t) * nnz, &m->coo_col));
   GKO_TRY(alloc(vs * nnz, &m->coo_val));
+  GKO_TRY(build_tile_starts(m.get(), ptr<int32_t>(csr->row_ptr), nnz, csr->plan.max_len, s));
   if (nnz > 0) {
     coo_rows_kernel<<<grid_for(nnz), 256, 0, s>>>(csr->n_rows, nnz, ptr<int32_t>(csr->row_ptr),
                                                    ptr<int32_t>(m->coo_row));
@@ -799,7 +850,9 @@ int gko_matrix_convert_to_hybrid(gko_matrix csr, int32_t ell_width, void* stream
   GKO_TRY(exclusive_scan(TailLen{ptr<int32_t>(csr->row_ptr), K}, n, ptr<int32_t>(tptr), &tail, s));
   const size_t vs = dtype_size(csr->dtype);
   m->coo_nnz = tail;
-  GKO_TRY(alloc(sizeof(int32_t) * tail, &m->coo_row));
+  const int32_t tail_len = std::max<int32_t>(0, csr->plan.max_len - K);  // longest row of the tail
+  GKO_TRY(alloc(sizeof(int32_t) * coo_row_words(n, tail, tail_len), &m->coo_row));
+  GKO_TRY(build_tile_starts(m.get(), ptr<int32_t>(tptr), tail, tail_len, s));
   GKO_TRY(alloc(sizeof(int32_t) * tail, &m->coo_col));
   GKO_TRY(alloc(vs * tail, &m->coo_val));
   if (tail > 0) {
@@ -859,6 +912,10 @@ int gko_matrix_convert_values(gko_matrix src, gko_dtype to, void* stream, gko_ma
   m->plan.merge_tiles = src->plan.merge_tiles;
   m->plan.seg_row = src->plan.seg_row;
   m->plan.seg_tiles = src->plan.seg_tiles;
+  m->plan.tile_start = src->plan.tile_start;
+  m->plan.tile_start_at = src->plan.tile_start_at;
+  m->plan.tiles = src->plan.tiles;
+  m->plan.tile_width = src->plan.tile_width;
   m->plan.coo_rb = src->plan.coo_rb;
   m->plan.coo_rb_n = src->plan.coo_rb_n;
   m->K = src->K;

@@ -12,15 +12,17 @@ size_t spmv_scratch_bytes(const gko_matrix_s* A) {
   switch (A->fmt) {
     case GKO_CSR:
       if (A->plan.kind == 2) return at * 2 * (size_t)((A->n_rows + A->nnz + 2047) / 2048 + 1);
+      if (A->plan.kind == 3 && A->plan.tiles) return 0;
       if (A->plan.kind == 3) return at * 2 * (size_t)((A->nnz + kCooTile - 1) / kCooTile + 1);
       return at * (size_t)A->plan.n_chunks;
     case GKO_ELL:
     case GKO_SELLP:
       return 0;
     case GKO_COO:
-      if (A->plan.kind == 1) return 0;
+      if (A->plan.kind == 1 || A->plan.tiles) return 0;
       return at * 2 * (size_t)((A->coo_nnz + kCooTile - 1) / kCooTile);
     case GKO_HYBRID:
+      if (A->plan.tiles) return 0;
       return at * 2 * (size_t)((A->coo_nnz + kCooTile - 1) / kCooTile);
   }
   return 0;

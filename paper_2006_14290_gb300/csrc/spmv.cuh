@@ -50,4 +50,24 @@ constexpr int kCooThreads = 128;
 constexpr int kCooItems = 8;
 constexpr int kCooTile = kCooThreads * kCooItems;
 
+// Row-aligned tiles of W nonzeros (a multiple of 8, for 16-byte loads).  A
+// block's window is the kCooTile entries from t W on; W leaves room for the
+// rest of the tile's last row where rows are short, so the window nearly
+// always holds the whole tile.
+// Used where the longest row is at most kTileRowMax (one block adds what a
+// row has behind the window: with rows of 10,000 the power-law matrices took
+// 62-103 us instead of 54-79) and where the launch and the workspace that go
+// away are worth more than the overlapping windows and the stores' bounds:
+// up to kTileNnzMax nonzeros (COO on 64^2 11.6 -> 8.8 us, CSR on 5,000
+// power-law rows 14.4 -> 10.2; 27-point COO on 128^3, 55.7 M, 189 -> 197), or
+// rows of kTileRowMean on average, few ends to bound (banded, 39.4 M: 144.6
+// -> 139.6).
+constexpr int32_t kTileRowMax = 2048;
+constexpr int64_t kTileNnzMax = 1 << 23;
+constexpr int64_t kTileRowMean = 32;
+inline int32_t tile_width_for(int32_t max_len) {
+  const int32_t room = max_len < 64 ? max_len : 64;
+  return (kCooTile - room) / 8 * 8;
+}
+
 }  // namespace gko

@@ -422,7 +422,8 @@ __global__ void __launch_bounds__(kRbThreads) coo_rowblock_kernel(CsrArgs<VT, XT
 // walk starts from `head` rather than from zero: 0 + t is a real FP64 add
 // (signed zeros keep the compiler from folding it), and FP64 instructions
 // co-limit these kernels.  The tile's last-segment sum goes to carry[2*tile+1], and also
-// to carry[2*tile] when no thread ended a row.
+// to carry[2*tile] when no thread ended a row; want_carry = false leaves both
+// out.
 // Every warp holding a row end (short rows): each ending thread walks back
 // through shared memory, about one FP64 add per thread in total.  A warp
 // without a row end (a row longer than a warp's entries) would make some
@@ -432,7 +433,7 @@ __global__ void __launch_bounds__(kRbThreads) coo_rowblock_kernel(CsrArgs<VT, XT
 // reproducible.
 template <typename AT, int NT>
 __device__ __forceinline__ void tile_carries(AT tail, bool has_end, AT head, AT* s_tail, int* s_end, AT* carry,
-                                             int64_t tile, AT& total, bool& from_before) {
+                                             int64_t tile, AT& total, bool& from_before, bool want_carry = true) {
   constexpr int NW = NT / 32;
   __shared__ AT s_wv[NW];
   __shared__ int s_wf[NW];
@@ -453,7 +454,7 @@ __device__ __forceinline__ void tile_carries(AT tail, bool has_end, AT head, AT*
         }
       }
     }
-    if (t == 0) {
+    if (t == 0 && want_carry) {
       AT tv = s_tail[NT - 1];
       bool any_end = s_end[NT - 1] != 0;
       for (int u = NT - 2; u >= 0 && !any_end; --u) {
@@ -505,7 +506,7 @@ __device__ __forceinline__ void tile_carries(AT tail, bool has_end, AT head, AT*
     total = ve + head;
     from_before = !fe;
   }
-  if (t == NT - 1) {
+  if (t == NT - 1 && want_carry) {
     const AT tv = f ? v : cw + v;
     if (!(f || cf)) carry[2 * tile] = tv;
     carry[2 * tile + 1] = tv;
@@ -961,12 +962,13 @@ constexpr int coo_min_blocks() {
 // end here are stored now.  FULL: all IPT entries are present (every thread
 // of every tile but the last), so the entry guards and the next-row choice
 // are compile-time.  The row-end bookkeeping is written as selects around a
-// predicated store (measured the same as the branchy form).
+// predicated store (measured the same as the branchy form).  Rows that end
+// outside entries lo .. hi - 1 are another tile's: not stored, first_row -1.
 template <bool FULL, bool ACCUM, bool PLAIN, int IPT, typename VT, typename XT, typename AT>
 __device__ __forceinline__ void coo_thread_pass(const CooArgs<VT, XT>& a, const int32_t (&rows)[IPT],
                                                 const int32_t (&cols)[IPT], const VT (&vals)[IPT], int my,
                                                 int32_t next_row, AT& run, AT& first_sum, int32_t& first_row,
-                                                int& nends) {
+                                                int& nends, int lo = 0, int hi = IPT) {
 #pragma unroll
   for (int u = 0; u < IPT; ++u) {
     if (FULL || u < my) {
@@ -974,10 +976,11 @@ __device__ __forceinline__ void coo_thread_pass(const CooArgs<VT, XT>& a, const 
       run = madd(to_acc(vals[u]), to_acc(ld_vec(a.x + cols[u])), run);
       const int32_t nr = FULL ? (u + 1 < IPT ? rows[u + 1] : next_row) : (u + 1 < my ? rows[u + 1] : next_row);
       const bool e = r != nr;
-      if (e && nends > 0) coo_store(a.y, r, run, a.alpha, a.beta, ACCUM, PLAIN);
+      const bool mine = u >= lo && u < hi;
+      if (e && nends > 0 && mine) coo_store(a.y, r, run, a.alpha, a.beta, ACCUM, PLAIN);
       const bool f = e && nends == 0;
       first_sum = f ? run : first_sum;
-      first_row = f ? r : first_row;
+      first_row = f ? (mine ? r : -1) : first_row;
       nends += e ? 1 : 0;
       run = e ? AT(0) : run;
     }
@@ -1137,6 +1140,142 @@ inline void coo_launch(const CooArgs<VT, XT>& a, acc_t<VT>* carry, const int* ga
   coo_fixup_kernel<VT, XT, ACCUM><<<fg, 256, 0, s>>>(a.nnz, tiles, a.row, carry, a.y, a.alpha, a.beta, gate);
 }
 
+// ------------------------------------------------- row-aligned tiles --
+//
+// The segmented pass without anything between blocks: tile t owns the rows
+// that start at nonzeros [t W, (t+1) W), so no partial sum leaves its block,
+// and the fix-up launch and the carries' workspace, which a call would have
+// to allocate, go away.  The block runs the pass over the kCooTile entries
+// from t W on as the kernels with carries do, whatever rows they belong to;
+// only the stores ask for the tile's own entries [s0, s1), so that neither
+// the loads nor the gathers wait for the tile's bounds (windows that start at
+// s0, or gathers that skip foreign entries, took banded COO from 145 to
+// 210-230 us).  The entries of a longer last row behind the window are added
+// by the whole block at the end.  Which matrices take tiles: spmv.cuh.
+
+// Sum over the block, valid in thread 0.
+template <typename AT>
+__device__ __forceinline__ AT tile_block_sum(AT v) {
+  __shared__ AT red[kCooThreads / 32];
+  v = subwarp_sum<32>(v, 0xffffffffu);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  AT s = red[0];
+#pragma unroll
+  for (int i = 1; i < kCooThreads / 32; ++i) s += red[i];
+  return s;
+}
+
+// Entries [k, k1) of one row, strided over the block.
+template <typename VT, typename XT>
+__device__ __forceinline__ acc_t<VT> tile_rest(const int32_t* col, const VT* val, const XT* x, int64_t k, int64_t k1) {
+  acc_t<VT> v = acc_t<VT>(0);
+  k += threadIdx.x;
+  for (; k + 3 * kCooThreads < k1; k += 4 * kCooThreads) {
+    int32_t c[4];
+    VT w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      c[u] = ld_stream(col + k + u * kCooThreads);
+      w[u] = ld_stream(val + k + u * kCooThreads);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v = madd(to_acc(w[u]), to_acc(ld_vec(x + c[u])), v);
+  }
+  for (; k < k1; k += kCooThreads) v = madd(to_acc(ld_stream(val + k)), to_acc(ld_vec(x + ld_stream(col + k))), v);
+  return v;
+}
+
+template <typename VT, typename XT, bool ACCUM, bool PLAIN>
+__global__ void __launch_bounds__(kCooThreads, coo_min_blocks<VT>())
+    coo_tile_kernel(CooArgs<VT, XT> a, const int32_t* __restrict__ start, int32_t width, const int* gate) {
+  using AT = acc_t<VT>;
+  constexpr int IPT = kCooItems;
+  __shared__ AT s_tail[kCooThreads];
+  __shared__ int s_end[kCooThreads];
+  __shared__ AT s_carry[2];
+  if (gated(gate)) return;
+  prefetch_slice_l2(a.x, sizeof(XT) * (size_t)a.n_cols, kXPrefetchBlocks);
+  const int t = threadIdx.x;
+  const int64_t base = (int64_t)blockIdx.x * width;
+  const int cnt = (int)min((int64_t)kCooTile, a.nnz - base);
+  const int j0 = t * IPT;
+  const int my = max(0, min(IPT, cnt - j0));
+  int32_t rows[IPT];
+  int32_t cols[IPT];
+  VT vals[IPT];
+  if (my == IPT) {
+    load8_i32(a.row + base + j0, rows);
+    load8_i32(a.col + base + j0, cols);
+    Load8<VT>::run(a.val + base + j0, vals);
+  } else {
+#pragma unroll
+    for (int u = 0; u < IPT; ++u) {
+      const int64_t k = base + j0 + u;
+      rows[u] = u < my ? a.row[k] : INT_MAX;
+      cols[u] = u < my ? a.col[k] : 0;
+      vals[u] = u < my ? a.val[k] : VT(0);
+    }
+  }
+  const int32_t s0 = __ldg(start + blockIdx.x), s1 = __ldg(start + blockIdx.x + 1);
+  // row of the entry after this thread's last one, -1 after the matrix's last
+  const int32_t nb = __shfl_down_sync(0xffffffffu, my > 0 ? rows[0] : INT_MAX, 1);
+  int32_t next_row;
+  if (j0 + IPT < cnt)
+    next_row = (t & 31) != 31 ? nb : a.row[base + j0 + IPT];
+  else
+    next_row = (base + cnt < a.nnz) ? a.row[base + cnt] : -1;
+  if (!ACCUM && base == 0 && t == 0 && my > 0) coo_empty_rows(a.y, 0, (int64_t)rows[0], a.beta);
+
+  const int lo = s0 - (int32_t)(base + j0), hi = s1 - (int32_t)(base + j0);  // the tile's entries u = lo .. hi - 1
+  AT run = AT(0), first_sum = AT(0);
+  int32_t first_row = -1;
+  int nends = 0;
+  if (my == IPT)
+    coo_thread_pass<true, ACCUM, PLAIN>(a, rows, cols, vals, my, next_row, run, first_sum, first_row, nends, lo, hi);
+  else
+    coo_thread_pass<false, ACCUM, PLAIN>(a, rows, cols, vals, my, next_row, run, first_sum, first_row, nends, lo, hi);
+  // rows without entries after a row end here (see coo_kernel)
+  const int32_t n_rows32 = (int32_t)a.n_rows;
+  if (!ACCUM && my > 0 && (next_row < 0 ? n_rows32 : next_row) - rows[0] > nends) {
+#pragma unroll 1
+    for (int u = max(lo, 0); u < min(hi, my); ++u) {
+      const int64_t k = base + j0 + u;
+      const int32_t r = a.row[k];
+      const int32_t nr = (u + 1 < my) ? a.row[k + 1] : next_row;
+      const int32_t gap_end = nr < 0 ? n_rows32 : nr;
+      if (r != nr && r + 1 < gap_end) coo_empty_rows(a.y, (int64_t)r + 1, (int64_t)gap_end, a.beta);
+    }
+  }
+  const bool beyond = s1 > base + kCooTile && s0 < s1;  // the tile's last row goes on behind the window
+  AT total;
+  bool from_before;
+  tile_carries<AT, kCooThreads>(run, nends > 0, first_sum, s_tail, s_end, s_carry, 0, total, from_before, beyond);
+  if (nends > 0 && first_row >= 0) coo_store(a.y, first_row, total, a.alpha, a.beta, ACCUM, PLAIN);
+  if (beyond) {
+    const AT rest = tile_block_sum(tile_rest(a.col, a.val, a.x, base + kCooTile, s1));
+    if (t == 0) {
+      const int32_t r = a.row[s1 - 1], nr = s1 < a.nnz ? a.row[s1] : n_rows32;
+      coo_store(a.y, r, s_carry[1] + rest, a.alpha, a.beta, ACCUM, PLAIN);
+      if (!ACCUM) coo_empty_rows(a.y, (int64_t)r + 1, (int64_t)nr, a.beta);
+    }
+  }
+}
+
+template <typename VT, typename XT, bool ACCUM>
+inline cudaError_t coo_tile_launch(const CooArgs<VT, XT>& a, const CsrPlan& p, const int* gate, cudaStream_t s) {
+  const int32_t* start = ptr<int32_t>(p.tile_start) + p.tile_start_at;
+  const unsigned g = (unsigned)p.tiles;
+  if constexpr (!ACCUM) {
+    if (a.plain) {
+      coo_tile_kernel<VT, XT, false, true><<<g, kCooThreads, 0, s>>>(a, start, p.tile_width, gate);
+      return cudaGetLastError();
+    }
+  }
+  coo_tile_kernel<VT, XT, ACCUM, false><<<g, kCooThreads, 0, s>>>(a, start, p.tile_width, gate);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------- nonzero-split CSR --
 //
 // Nonzero-split CSR (skewed matrices): the nonzeros are cut into tiles of
@@ -1156,7 +1295,8 @@ constexpr int kSegRpCap = 2048;
 template <bool FULL, bool PLAIN, typename VT, typename XT, typename AT, typename RPV>
 __device__ __forceinline__ void csr_seg_pass(const CsrArgs<VT, XT>& a, const int32_t (&cols)[kCooItems],
                                              const VT (&vals)[kCooItems], int my, int32_t k0, const RPV& rpv,
-                                             int32_t r, AT& run, AT& first_sum, int32_t& first_row, int& nends) {
+                                             int32_t r, AT& run, AT& first_sum, int32_t& first_row, int& nends,
+                                             int lo = 0, int hi = kCooItems) {
   const int32_t n32 = (int32_t)a.n;
   int32_t nb = rpv(r + 1);  // one past the last nonzero of row r
 #pragma unroll
@@ -1165,10 +1305,11 @@ __device__ __forceinline__ void csr_seg_pass(const CsrArgs<VT, XT>& a, const int
       run = madd(to_acc(vals[u]), to_acc(ld_vec(a.x + cols[u])), run);
       const int32_t k1 = k0 + u + 1;
       if (k1 == nb) {  // row r ends at this entry
+        const bool mine = u >= lo && u < hi;  // else another tile's row
         if (nends == 0) {
           first_sum = run;
-          first_row = r;
-        } else {
+          first_row = mine ? r : -1;
+        } else if (mine) {
           coo_store(a.y, r, run, a.alpha, a.beta, false, PLAIN);
         }
         ++nends;
@@ -1177,7 +1318,7 @@ __device__ __forceinline__ void csr_seg_pass(const CsrArgs<VT, XT>& a, const int
         ++r;
         nb = r < n32 ? rpv(r + 1) : INT_MAX;
         while (nb == k1) {
-          coo_empty_rows(a.y, (int64_t)r, (int64_t)r + 1, a.beta);
+          if (mine) coo_empty_rows(a.y, (int64_t)r, (int64_t)r + 1, a.beta);
           ++r;
           nb = r < n32 ? rpv(r + 1) : INT_MAX;
         }
@@ -1275,6 +1416,85 @@ __global__ void __launch_bounds__(256)
       if (!(u + 1 < tiles && seg_row[u + 1] == r)) break;  // row r ends in tile u
     }
     a.y[r] = (XT)finish_row(a.y, r, s, a.alpha, a.beta, a.plain);
+  }
+}
+
+// The nonzero split in row-aligned tiles (see the row-aligned COO tiles).
+// seg_row[t] is the row of nonzero t W: the tile's entries start there if the
+// row does, else with the next row, and end likewise at the next tile's.  Rows
+// without nonzeros belong to the tile of the row end before them.
+template <typename VT, typename XT, bool PLAIN>
+__global__ void __launch_bounds__(kCooThreads, coo_min_blocks<VT>())
+    csr_tile_kernel(CsrArgs<VT, XT> a, int64_t nnz, const int32_t* __restrict__ seg_row, int32_t width,
+                    const int* gate) {
+  using AT = acc_t<VT>;
+  __shared__ int32_t s_rp[kSegRpCap + 3];
+  __shared__ AT s_tail[kCooThreads];
+  __shared__ int s_end[kCooThreads];
+  __shared__ AT s_carry[2];
+  if (gated(gate)) return;
+  prefetch_slice_l2(a.x, sizeof(XT) * (size_t)a.n_cols, kXPrefetchBlocks);
+  const int t = threadIdx.x;
+  const int64_t base = (int64_t)blockIdx.x * width;
+  const int cnt = (int)min((int64_t)kCooTile, nnz - base);
+  const int j0 = t * kCooItems;
+  const int my = max(0, min(kCooItems, cnt - j0));
+  int32_t cols[kCooItems];
+  VT vals[kCooItems];
+  if (my == kCooItems) {
+    load8_i32(a.col + base + j0, cols);
+    Load8<VT>::run(a.val + base + j0, vals);
+  } else {
+#pragma unroll
+    for (int u = 0; u < kCooItems; ++u) {
+      cols[u] = u < my ? a.col[base + j0 + u] : 0;
+      vals[u] = u < my ? a.val[base + j0 + u] : VT(0);
+    }
+  }
+  const int32_t ra = __ldg(seg_row + blockIdx.x), rb = __ldg(seg_row + blockIdx.x + 1);
+  const int32_t last = min(rb + 2, (int32_t)a.n);  // row pointers ra .. last
+  const bool staged = last - ra + 1 <= kSegRpCap + 3;
+  if (staged)
+    for (int i = t; i <= last - ra; i += kCooThreads) s_rp[i] = __ldg(a.rp + ra + i);
+  __syncthreads();
+  const auto rpv = [&](int32_t r) -> int32_t { return staged && r <= last ? s_rp[r - ra] : __ldg(a.rp + r); };
+  if (base == 0 && t == 0) coo_empty_rows(a.y, 0, (int64_t)ra, a.beta);
+  const int64_t s0 = rpv(ra) == base ? base : rpv(ra + 1);
+  const int64_t s1 = base + width >= nnz ? nnz : rpv(rb) == base + width ? base + width : rpv(rb + 1);
+  // the last row at or before rb that starts at or before entry k
+  const auto row_at = [&](int32_t k) -> int32_t {
+    int32_t l = ra, h = rb;
+    while (l < h) {
+      const int32_t mid = l + (h - l + 1) / 2;
+      if (rpv(mid) <= k) l = mid;
+      else h = mid - 1;
+    }
+    return l;
+  };
+  const int32_t k0 = (int32_t)(base + j0);
+  AT run = AT(0), first_sum = AT(0);
+  int32_t first_row = -1;
+  int nends = 0;
+  if (my > 0) {
+    const int32_t r = row_at(k0);
+    const int lo = (int)(s0 - k0), hi = (int)(s1 - k0);  // the tile's entries u = lo .. hi - 1
+    if (my == kCooItems)
+      csr_seg_pass<true, PLAIN>(a, cols, vals, my, k0, rpv, r, run, first_sum, first_row, nends, lo, hi);
+    else
+      csr_seg_pass<false, PLAIN>(a, cols, vals, my, k0, rpv, r, run, first_sum, first_row, nends, lo, hi);
+  }
+  const bool beyond = s1 > base + kCooTile && s0 < s1;  // the tile's last row goes on behind the window
+  AT total;
+  bool from_before;
+  tile_carries<AT, kCooThreads>(run, nends > 0, first_sum, s_tail, s_end, s_carry, 0, total, from_before, beyond);
+  if (nends > 0 && first_row >= 0) coo_store(a.y, first_row, total, a.alpha, a.beta, false, PLAIN);
+  if (beyond) {
+    const AT rest = tile_block_sum(tile_rest(a.col, a.val, a.x, base + kCooTile, s1));
+    if (t == 0) {
+      int32_t r = row_at((int32_t)(s1 - 1));
+      coo_store(a.y, r, s_carry[1] + rest, a.alpha, a.beta, false, PLAIN);
+      for (++r; r < (int32_t)a.n && rpv(r + 1) == s1; ++r) coo_empty_rows(a.y, (int64_t)r, (int64_t)r + 1, a.beta);
+    }
   }
 }
 
@@ -1426,6 +1646,14 @@ struct SpmvImpl {
         GKO_TRY_CUDA(cudaGetLastError());
         return GKO_OK;
       }
+      if (A->plan.tiles) {
+        const CsrArgs<VT, XT> ta = csr_args(A, x, y, alpha, beta);
+        auto kern = ta.plain ? csr_tile_kernel<VT, XT, true> : csr_tile_kernel<VT, XT, false>;
+        kern<<<(unsigned)A->plan.tiles, kCooThreads, 0, s>>>(ta, A->nnz, ptr<int32_t>(A->plan.seg_row),
+                                                             A->plan.tile_width, gate);
+        GKO_TRY_CUDA(cudaGetLastError());
+        return GKO_OK;
+      }
       const int64_t tiles = (A->nnz + kCooTile - 1) / kCooTile;
       AT* carry = static_cast<AT*>(scratch);
       const CsrArgs<VT, XT> ca = csr_args(A, x, y, alpha, beta);
@@ -1526,6 +1754,12 @@ struct SpmvImpl {
     AT* carry = static_cast<AT*>(scratch);
     CooArgs<VT, XT> a{A->n_rows, A->n_cols, nnz, ptr<int32_t>(A->coo_row), ptr<int32_t>(A->coo_col),
                       ptr<VT>(A->coo_val), x, y, alpha, beta, alpha == AT(1) && beta == AT(0)};
+    if (A->plan.tiles) {
+      const cudaError_t e = accum ? coo_tile_launch<VT, XT, true>(a, A->plan, gate, s)
+                                  : coo_tile_launch<VT, XT, false>(a, A->plan, gate, s);
+      GKO_TRY_CUDA(e);
+      return GKO_OK;
+    }
     if (accum)
       coo_launch<VT, XT, true>(a, carry, gate, s);
     else

@@ -62,8 +62,6 @@ extern "C" int gko_spmv_coo_noalloc(const double* alpha, gko_matrix A, const dou
   if (A->n_rows > 0 && !y) return fail(GKO_INVALID_ARG, "null y");
   if (A->coo_nnz > 0 && !x) return fail(GKO_INVALID_ARG, "null x");
   if (A->n_rows == 0) return GKO_OK;
-  double* carry = nullptr;
-  GKO_TRY(noalloc_scratch(&carry));
   cudaStream_t s = (cudaStream_t)stream;
   const double a = *alpha, b = *beta;
   const int64_t nnz = A->coo_nnz;
@@ -73,11 +71,18 @@ extern "C" int gko_spmv_coo_noalloc(const double* alpha, gko_matrix A, const dou
     GKO_TRY_CUDA(cudaGetLastError());
     return GKO_OK;
   }
+  CooArgs<double, double> args{A->n_rows, A->n_cols, nnz, ptr<int32_t>(A->coo_row), ptr<int32_t>(A->coo_col),
+                               ptr<double>(A->coo_val), x, y, a, b, a == 1.0 && b == 0.0};
+  if (A->plan.tiles) {  // row-aligned tiles: no carries
+    const cudaError_t e = coo_tile_launch<double, double, false>(args, A->plan, nullptr, s);
+    GKO_TRY_CUDA(e);
+    return GKO_OK;
+  }
+  double* carry = nullptr;
+  GKO_TRY(noalloc_scratch(&carry));
   // Every carry slot the fix-up reads is written earlier in the same call, so
   // nothing needs clearing; calls that overlap on the GPU share the array
   // and race.
-  CooArgs<double, double> args{A->n_rows, A->n_cols, nnz, ptr<int32_t>(A->coo_row), ptr<int32_t>(A->coo_col),
-                               ptr<double>(A->coo_val), x, y, a, b, a == 1.0 && b == 0.0};
   coo_launch<double, double, false>(args, carry, nullptr, s);
   GKO_TRY_CUDA(cudaGetLastError());
   return GKO_OK;

@@ -1,0 +1,56 @@
+"""COO, hybrid and nonzero-split SpMV in row-aligned tiles at the edges of the
+tiles and of the rule that selects them, against the oracle."""
+import numpy as np
+import pytest
+
+from gpu_util import bf16_round, check_spmv_f32, check_spmv_f64, dev, host
+from paper_2006_14290_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def cases():
+    rng = np.random.default_rng(77)
+    yield "one_entry", [0, 0, 1, 0]
+    yield "row_fills_window", [1024, 1, 1023, 3]
+    # rows that end on, one before and one after every tile (W = 960 with rows of 64 and more) and window
+    yield "tile_ends", [960, 960, 959, 1, 961, 0, 0, 958, 2, 64, 896, 0] * 7
+    yield "beyond_window", [5, 0, 1500, 0, 0, 3] * 40 + [2048, 0, 2048, 1, 2047]  # whole tiles inside a row
+    yield "longest_tiled", [2048] * 20
+    yield "too_long", [7] * 500 + [2049] + [7] * 500  # carries
+    yield "empty_runs", [0] * 5000 + [3] * 200 + [0] * 4000 + [9, 0] * 300 + [0] * 3000
+    yield "short", list(rng.integers(0, 5, 9000))
+    yield "skewed", list(np.minimum(rng.zipf(2.0, 4000), 2000))
+    yield "tail_of_one", [8] * 119 + [7] + [1]
+
+
+CASES = [(n, I.rows_csr(L, 3000, np.random.default_rng(len(L)))) for n, L in cases()]
+
+
+@pytest.mark.parametrize("name,A", CASES, ids=[c[0] for c in CASES])
+@pytest.mark.parametrize("fmt", ["coo", "split", "hybrid0", "hybrid2"])
+@pytest.mark.parametrize("dt", ["f64", "f32", "bf16"])
+def test_tiles_match_oracle(gko, name, A, fmt, dt):
+    G = gko
+    M = G.from_csr(A)
+    if dt != "f64":
+        M = G.gko_matrix_convert_values(M, G.F32 if dt == "f32" else G.BF16)
+    if fmt == "coo":
+        M = G.gko_matrix_convert_to_coo(M)
+    elif fmt == "split":
+        M.set_plan(3, 1, 1, 1024)
+    else:
+        M = G.gko_matrix_convert_to_hybrid(M, int(fmt[-1]))
+    rng = np.random.default_rng(5)
+    x, y0 = rng.uniform(-1, 1, A.n_cols), rng.uniform(-1, 1, A.n_rows)
+    for alpha, beta in [(1.0, 0.0), (-0.75, 1.5)]:
+        if dt == "f64":
+            yd = dev(y0 if beta else np.full(A.n_rows, np.nan))
+            G.gko_spmv(alpha, M, dev(x), beta, yd)
+            check_spmv_f64(host(yd), A, x, alpha, beta, y0)
+        else:
+            x32, v = x.astype(np.float32), A.val.astype(np.float32).astype(np.float64)
+            yd = dev(y0, np.float32)
+            G.gko_spmv(alpha, M, dev(x32), beta, yd)
+            check_spmv_f32(host(yd), A, x32.astype(np.float64), alpha, beta, y0.astype(np.float32).astype(np.float64),
+                           v if dt == "f32" else bf16_round(A.val))
