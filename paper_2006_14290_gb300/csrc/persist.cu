@@ -81,6 +81,8 @@ int launch(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const Solv
   a.b = b;
   a.x = x;
   a.d = static_cast<const T*>(sp.minv);
+  a.bj = static_cast<const T*>(sp.bj);
+  a.bs = sp.bs;
   a.rel_tol = sp.rel_tol;
   a.maxit = sp.maxit;
   a.check_true = sp.check_true;
@@ -124,19 +126,30 @@ int run(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSp
   // where none does, the first that reads its entries from the matrix
   auto smem_of = [&](const PkShape& h, bool st) {
     const size_t rb = (size_t)h.nt * h.rpt;
-    return (st ? K * rb * (sizeof(VT) + sizeof(int32_t)) : 0) + (h.mode == kPkCluster ? kPkClusterVecs * rb * sizeof(T) : 0);
+    return (st ? K * rb * (sizeof(VT) + sizeof(int32_t)) : 0) +
+           ((h.mode == kPkCluster ? kPkClusterVecs : 0) + (sp.bj ? 1 : 0)) * rb * sizeof(T);
   };
   auto blocks_of = [&](const PkShape& h) { return (n + h.nt * h.rpt - 1) / (h.nt * h.rpt); };
   auto covers = [&](const PkShape& h) {
     return blocks_of(h) <= (h.mode == kPkCluster ? kPkCluster16 : std::min(sm_count(), kPkMaxBlocks));
   };
-  for (bool staged : {true, false})
-    for (int i = staged ? 0 : kPkFirstGlobal; i < kPkNShapes; ++i) {
-      if (!covers(kPkShapes[i]) || smem_of(kPkShapes[i], staged) > kPkSmemMax) continue;
-      const int rc = launch<T, VT>(A, b, x, x_zero, sp, s, out, i, staged, (int)blocks_of(kPkShapes[i]), K,
-                                   smem_of(kPkShapes[i], staged));
+  const bool published = sp.solver == 1 && sp.bj;  // no kPkFly
+  auto attempt = [&](int i, bool staged) -> int {
+    const PkShape& h = kPkShapes[i];
+    if (!covers(h) || (published && h.mode == kPkFly) || smem_of(h, staged) > kPkSmemMax) return GKO_NOT_SUPPORTED;
+    return launch<T, VT>(A, b, x, x_zero, sp, s, out, i, staged, (int)blocks_of(h), K, smem_of(h, staged));
+  };
+  for (bool staged : {true, false}) {
+    const int first = staged ? 0 : kPkFirstGlobal;
+    for (int i = first; i <= kPkLastGlobal; ++i) {
+      if (published && staged && kPkShapes[i].mode == kPkFly) {  // its published twin
+        const int rc = attempt(i + kPkTwin, true);
+        if (rc != GKO_NOT_SUPPORTED) return rc;
+      }
+      const int rc = attempt(i, staged);
       if (rc != GKO_NOT_SUPPORTED) return rc;
     }
+  }
   return GKO_NOT_SUPPORTED;
 }
 
@@ -146,7 +159,8 @@ int persist_solve(const gko_matrix_s* A, const double* b, void* x, bool x_zero, 
                   SolveOut* out) {
   // CSR under the row-block plan (regular rows: other plans keep their SpMV
   // kernels), ELL and SELL-P; reliable updates for BiCGSTAB only
-  if (sp.solver > 1 || sp.bj || A->n_rows <= 0 || A->n_rows > kSmallRows) return GKO_NOT_SUPPORTED;
+  if (sp.solver > 1 || A->n_rows <= 0 || A->n_rows > kSmallRows) return GKO_NOT_SUPPORTED;
+  if (sp.bj && (sp.bs & (sp.bs - 1))) return GKO_NOT_SUPPORTED;  // diagonal blocks end with thread blocks
   if (!(A->fmt == GKO_CSR && A->plan.kind == 1) && A->fmt != GKO_ELL && A->fmt != GKO_SELLP) return GKO_NOT_SUPPORTED;
   if (sp.rel && (sp.solver != 1 || sp.rel->A64->fmt != A->fmt)) return GKO_NOT_SUPPORTED;
   int dev = 0, coop = 0;

@@ -63,6 +63,8 @@ struct PkArgs {
   const double* b;  // right-hand side (reliable updates: the initial residual)
   T* x;
   const T* d;       // Jacobi inverse diagonal, or null
+  const T* bj;      // block-Jacobi inverse blocks (n x bs), or null; bs a power of two up to 32
+  int bs;
   double rel_tol;
   int maxit;
   int check_true;
@@ -435,6 +437,37 @@ struct PkRows {
   }
 };
 
+// z = M^-1 v for the thread's rows: Jacobi (d_j), block-Jacobi (the rows of a
+// diagonal block are consecutive threads of this block; v goes through shared
+// memory, the inverse block's row is read from L2) or none.
+template <typename T, typename VT, int NT, int RPT>
+struct PkPrecond {
+  T* s;  // NT * RPT entries, block-Jacobi only
+  __device__ __forceinline__ void apply(const PkArgs<T, VT>& a, const int32_t (&row)[RPT], const T (&d)[RPT],
+                                        const T (&v)[RPT], T (&z)[RPT]) const {
+    if (a.bj) {
+      pk_sync<NT>();
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) s[threadIdx.x + j * NT] = v[j];
+      pk_sync<NT>();
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) {
+        const int first = (int)threadIdx.x & -a.bs;  // thread of the diagonal block's first row
+        const int32_t base = row[j] - ((int)threadIdx.x - first);
+        const int nb = row[j] < 0 ? 0 : min(a.bs, a.n - base);
+        const T* B = a.bj + (int64_t)max(row[j], 0) * a.bs;
+        T t = T(0);
+#pragma unroll 8
+        for (int k = 0; k < nb; ++k) t = madd(__ldg(B + k), s[first + j * NT + k], t);
+        z[j] = t;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) z[j] = a.d ? d[j] * v[j] : v[j];
+    }
+  }
+};
+
 // ----------------------------------------------------------------- CG --
 
 template <typename T, typename VT, int NT, int RPT, int MODE, bool ST>
@@ -447,14 +480,17 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
   vec.init(a, smem_raw);
   constexpr int X = decltype(vec)::kX;
   PkRows<T, VT, NT, RPT, ST> rows;
-  rows.init(a, smem_raw + (MODE == kPkCluster ? kPkClusterVecs * NT * RPT * sizeof(T) : 0));
+  // shared memory: cluster vectors, block-Jacobi's vector, entries
+  unsigned char* sm = smem_raw + (MODE == kPkCluster ? kPkClusterVecs * NT * RPT * sizeof(T) : 0);
+  const PkPrecond<T, VT, NT, RPT> pre{reinterpret_cast<T*>(sm)};
+  rows.init(a, sm + (a.bj ? NT * RPT * sizeof(T) : 0));
   if constexpr (MODE == kPkCluster) {
     // no tag set; every block's slots are clear before a peer writes them
     for (int i = threadIdx.x; i < 2 * kPkCluster16 * 4; i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
     pk_cluster_barrier();
   }
   unsigned seq = 0;
-  const bool pc = a.d != nullptr;
+  const bool pc = a.d != nullptr || a.bj != nullptr;
   // vector 0: FLY z = M^-1 r, else p; FLY: vectors 1 and 2 p, alternating
   struct Zp {
     T z, p;
@@ -462,7 +498,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
   auto one = [](T v) { return v; };
   auto at = [&](int k) { return [&vec, k](int32_t c) { return vec.get(k, c); }; };
   auto x0 = [&](int32_t c) { return __ldcg(a.x + c); };
-  T xj[RPT], rj[RPT], pj[RPT], dj[RPT];
+  T xj[RPT], rj[RPT], pj[RPT], dj[RPT], zj[RPT];
   double v3[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int j = 0; j < RPT; ++j) {
@@ -472,20 +508,21 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
     if (i < 0) continue;
     const double bi = a.b[i];
     if (!a.x_zero) xj[j] = a.x[i];
-    if (pc) dj[j] = a.d[i];
+    if (a.d) dj[j] = a.d[i];
     // staged entries are this thread's own: no barrier needed to read them
     rj[j] = a.x_zero ? (T)bi : (T)(bi - wd((T)rows.template dot<U>(a, j, x0, one)));
-    const T zi = pc ? dj[j] * rj[j] : rj[j];
-    if (FLY) {
-      vec.put(0, i, zi);
-      vec.put(2, i, T(0));  // p_old of the first iteration
-    } else {
-      pj[j] = zi;
-      vec.put(0, i, zi);
-    }
     v3[0] += bi * bi;
     v3[1] += wd(rj[j]) * wd(rj[j]);
-    v3[2] += wd(rj[j]) * wd(zi);
+  }
+  pre.apply(a, rows.row, dj, rj, zj);
+#pragma unroll
+  for (int j = 0; j < RPT; ++j) {
+    const int32_t i = rows.row[j];
+    if (i < 0) continue;
+    vec.put(0, i, zj[j]);
+    if (FLY) vec.put(2, i, T(0));  // p_old of the first iteration
+    else pj[j] = zj[j];
+    v3[2] += wd(rj[j]) * wd(zj[j]);
   }
   // scalars of the recurrence: thread 0 of every block, the same in each
   double nb = 0.0, tol = 0.0, tol2 = 0.0, rho = 0.0, rho_prev = 0.0, rr_true = 0.0;
@@ -528,8 +565,10 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
       const int32_t i = rows.row[j];
       tj[j] = i >= 0 ? (T)(a.b[i] - wd((T)rows.template dot<U>(a, j, at(X), one))) : T(0);
       vt[0] += wd(tj[j]) * wd(tj[j]);
-      vt[1] += wd(tj[j]) * wd(pc ? dj[j] * tj[j] : tj[j]);
     }
+    pre.apply(a, rows.row, dj, tj, zj);
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) vt[1] += wd(tj[j]) * wd(zj[j]);
     return pk_step<NT, MODE, kPubNone, 2>(vt, sh, a.slots, a.err, seq, fin);
   };
   while (status == kRun) {
@@ -542,7 +581,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
         if (rows.row[j] < 0) continue;
-        pj[j] = bp(pj[j], pc ? dj[j] * rj[j] : rj[j]);
+        pj[j] = bp(pj[j], zj[j]);
         __stcg(pn + rows.row[j], pj[j]);
       }
 #pragma unroll
@@ -578,14 +617,18 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
       if (i < 0) continue;
       xj[j] = ax(pj[j], xj[j]);
       rj[j] = ar(qj[j], rj[j]);
-      const T zi = pc ? dj[j] * rj[j] : rj[j];
-      if (FLY) vec.put(0, i, zi);
       const double rw = wd(rj[j]);
       v2[0] = __fma_rn(rw, rw, v2[0]);
-      if (pc) v2[1] = __fma_rn(rw, wd(zi), v2[1]);
+    }
+    pre.apply(a, rows.row, dj, rj, zj);
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+      if (rows.row[j] < 0) continue;
+      if (FLY) vec.put(0, rows.row[j], zj[j]);
+      if (pc) v2[1] = __fma_rn(wd(rj[j]), wd(zj[j]), v2[1]);
     }
     double inv = 0.0;  // 1 / rho, formed while the sums travel
-    auto pre = [&] { inv = 1.0 / rho; };
+    auto ahead = [&] { inv = 1.0 / rho; };
     auto fin2 = [&](double rr, double rz, double* o) {
       o[0] = pk_meets(rr, tol, tol2) ? 1.0 : 0.0;
       // rz / rho: the product's error is removed with its exact residual
@@ -597,11 +640,11 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
     bool ok;
     if (pc) {
       ok = pk_step<NT, MODE, FLY ? kPubVec : kPubNone, 2>(v2, sh, a.slots, a.err, seq,
-                            [&](const double (&t)[2], double* o) { fin2(t[0], t[1], o); }, pre);
+                            [&](const double (&t)[2], double* o) { fin2(t[0], t[1], o); }, ahead);
     } else {
       const double w1[1] = {v2[0]};
       ok = pk_step<NT, MODE, FLY ? kPubVec : kPubNone, 1>(w1, sh, a.slots, a.err, seq,
-                            [&](const double (&t)[1], double* o) { fin2(t[0], t[0], o); }, pre);
+                            [&](const double (&t)[1], double* o) { fin2(t[0], t[0], o); }, ahead);
     }
     if (!ok) {
       status = -1;
@@ -633,7 +676,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
         rj[j] = tj[j];
-        if (FLY && rows.row[j] >= 0) vec.put(0, rows.row[j], pc ? dj[j] * rj[j] : rj[j]);
+        if (FLY && rows.row[j] >= 0) vec.put(0, rows.row[j], zj[j]);  // of t
       }
       if (FLY && !pk_step<NT, MODE, kPubVec, 0>(nullptr, sh, a.slots, a.err, seq, [](const double (&)[1], double*) {})) {
         status = -1;
@@ -647,7 +690,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
         if (rows.row[j] < 0) continue;
-        pj[j] = bp(pj[j], pc ? dj[j] * rj[j] : rj[j]);
+        pj[j] = bp(pj[j], zj[j]);
         vec.put(0, rows.row[j], pj[j]);
       }
       if (!pk_step<NT, MODE, kPubVec, 0>(nullptr, sh, a.slots, a.err, seq, [](const double (&)[1], double*) {})) {
@@ -692,14 +735,17 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
   vec.init(a, smem_raw);
   constexpr int X = decltype(vec)::kX;
   PkRows<T, VT, NT, RPT, ST> rows;
-  rows.init(a, smem_raw + (MODE == kPkCluster ? kPkClusterVecs * NT * RPT * sizeof(T) : 0));
+  // shared memory: cluster vectors, block-Jacobi's vector, entries
+  unsigned char* sm = smem_raw + (MODE == kPkCluster ? kPkClusterVecs * NT * RPT * sizeof(T) : 0);
+  const PkPrecond<T, VT, NT, RPT> pre{reinterpret_cast<T*>(sm)};
+  rows.init(a, sm + (a.bj ? NT * RPT * sizeof(T) : 0));
   if constexpr (MODE == kPkCluster) {
     // no tag set; every block's slots are clear before a peer writes them
     for (int i = threadIdx.x; i < 2 * kPkCluster16 * 4; i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
     pk_cluster_barrier();
   }
   unsigned seq = 0;
-  const bool pc = a.d != nullptr;
+  const bool pc = a.d != nullptr;  // FLY gatherers apply it
   const bool reliable = REL && a.val64 != nullptr;
   // FLY: r, p (two buffers), v (two buffers); else vec[0] = M^-1 p, vec[1] = M^-1 s
   T* rb = vec.g[0];
@@ -723,7 +769,7 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
     if (i < 0) continue;
     const double bi = a.b[i];
     if (!a.x_zero) xj[j] = a.x[i];
-    if (pc) dj[j] = a.d[i];
+    if (a.d) dj[j] = a.d[i];
     rj[j] = a.x_zero ? (T)bi : (T)(bi - wd((T)rows.template dot<U>(a, j, x0, one)));
     hj[j] = rj[j];
     if (FLY) {
@@ -817,10 +863,13 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
       phj[j] = T(0);
       if (i < 0) continue;
       pj[j] = bp(wv(vj[j], pj[j]), rj[j]);
-      phj[j] = pc ? dj[j] * pj[j] : pj[j];
       if (FLY) __stcg(pn + i, pj[j]);
-      else vec.put(0, i, phj[j]);
     }
+    pre.apply(a, rows.row, dj, pj, phj);
+    if constexpr (!FLY)
+#pragma unroll
+      for (int j = 0; j < RPT; ++j)
+        if (rows.row[j] >= 0) vec.put(0, rows.row[j], phj[j]);
     if constexpr (!FLY)
       if (!pk_step<NT, MODE, kPubVec, 0>(nullptr, sh, a.slots, a.err, seq, nothing)) {
         status = -1;
@@ -860,17 +909,21 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
     ++it;
     const Lin<T> ap = pk_lin<T>(sh.out[1]), av = pk_lin<T>(sh.out[2]);
     // ---- s, t = A M^-1 s, omega
-    T sj[RPT], tj[RPT];
+    T sj[RPT], tj[RPT], shj[RPT];
     double v3[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int j = 0; j < RPT; ++j) {
       sj[j] = T(0);
       if (rows.row[j] < 0) continue;
       sj[j] = av(vj[j], rj[j]);
-      if (!FLY) vec.put(1, rows.row[j], pc ? dj[j] * sj[j] : sj[j]);
       const double sw = wd(sj[j]);
       v3[2] = __fma_rn(sw, sw, v3[2]);
     }
+    pre.apply(a, rows.row, dj, sj, shj);
+    if constexpr (!FLY)
+#pragma unroll
+      for (int j = 0; j < RPT; ++j)
+        if (rows.row[j] >= 0) vec.put(1, rows.row[j], shj[j]);
     if constexpr (!FLY)
       if (!pk_step<NT, MODE, kPubVec, 0>(nullptr, sh, a.slots, a.err, seq, nothing)) {
         status = -1;
@@ -922,7 +975,7 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
       for (int j = 0; j < RPT; ++j) {
         const int32_t i = rows.row[j];
         if (i < 0) continue;
-        xj[j] = os(pc ? dj[j] * sj[j] : sj[j], ap(phj[j], xj[j]));
+        xj[j] = os(shj[j], ap(phj[j], xj[j]));
         rj[j] = ot(tj[j], sj[j]);
         if (FLY) vec.put(0, i, rj[j]);
         const double rw = wd(rj[j]);
@@ -1106,9 +1159,13 @@ struct PkShape {
 };
 constexpr PkShape kPkShapes[] = {
     {32, 1, kPkCluster}, {64, 1, kPkCluster}, {128, 1, kPkCluster}, {256, 1, kPkCluster}, {256, 2, kPkCluster},
-    {64, 1, kPkFly}, {128, 1, kPkFly}, {256, 1, kPkFly}, {512, 1, kPkFly}, {512, 2, kPkGrid}, {512, 4, kPkGrid}};
+    {64, 1, kPkFly}, {128, 1, kPkFly}, {256, 1, kPkFly}, {512, 1, kPkFly}, {512, 2, kPkGrid}, {512, 4, kPkGrid},
+    // BiCGSTAB with block-Jacobi, whose preconditioned directions no gatherer can recompute, instead of kPkFly
+    {64, 1, kPkGrid}, {128, 1, kPkGrid}, {256, 1, kPkGrid}, {512, 1, kPkGrid}};
 constexpr int kPkNShapes = sizeof(kPkShapes) / sizeof(kPkShapes[0]);
-constexpr int kPkFirstGlobal = 7;  // first shape with a variant that does not stage its entries
+// (unstaged variants: shapes kPkFirstGlobal to kPkLastGlobal)
+constexpr int kPkFirstGlobal = 7, kPkLastGlobal = 10;
+constexpr int kPkTwin = 6;  // from a kPkFly shape to the published one of its size
 
 // The kernel of a shape, with or without staging, or null; one translation
 // unit per solver and value type instantiates them (persist_*.cu).
@@ -1122,15 +1179,17 @@ PkKernel<T, VT> pk_bicg(int shape, bool staged);
   CASE(3, 256, 1, kPkCluster) CASE(4, 256, 2, kPkCluster) CASE(5, 64, 1, kPkFly)                     \
   CASE(6, 128, 1, kPkFly) CASE(7, 256, 1, kPkFly) CASE(8, 512, 1, kPkFly) CASE(9, 512, 2, kPkGrid)   \
   CASE(10, 512, 4, kPkGrid)
+#define GKO_PK_BLOCK_SHAPES(CASE)                                                                    \
+  CASE(11, 64, 1, kPkGrid) CASE(12, 128, 1, kPkGrid) CASE(13, 256, 1, kPkGrid) CASE(14, 512, 1, kPkGrid)
 #define GKO_PK_CG(SH, NT, RPT, MODE)                                                                  \
   if (shape == SH) {                                                                                 \
     if (staged) return pk_cg_kernel<T, VT, NT, RPT, MODE, true>;                                      \
-    if constexpr (SH >= kPkFirstGlobal) return pk_cg_kernel<T, VT, NT, RPT, MODE, false>;             \
+    if constexpr (SH >= kPkFirstGlobal && SH <= kPkLastGlobal) return pk_cg_kernel<T, VT, NT, RPT, MODE, false>;             \
   }
 #define GKO_PK_BICG(SH, NT, RPT, MODE)                                                                \
   if (shape == SH) {                                                                                 \
     if (staged) return pk_bicg_kernel<T, VT, NT, RPT, MODE, true, sizeof(T) == 4>;                    \
-    if constexpr (SH >= kPkFirstGlobal) return pk_bicg_kernel<T, VT, NT, RPT, MODE, false, sizeof(T) == 4>; \
+    if constexpr (SH >= kPkFirstGlobal && SH <= kPkLastGlobal) return pk_bicg_kernel<T, VT, NT, RPT, MODE, false, sizeof(T) == 4>; \
   }
 
 }  // namespace gko

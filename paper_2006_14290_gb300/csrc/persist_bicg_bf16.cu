@@ -8,6 +8,7 @@ PkKernel<float, __nv_bfloat16> pk_bicg<float, __nv_bfloat16>(int shape, bool sta
   using T = float;
   using VT = __nv_bfloat16;
   GKO_PK_SHAPES(GKO_PK_BICG)
+  GKO_PK_BLOCK_SHAPES(GKO_PK_BICG)
   return nullptr;
 }
 

@@ -145,3 +145,17 @@ def test_batch_mixed_widths_and_long_rows(gko):
         assert ro.status == 0 and np.linalg.norm(xi - xo) <= 1e-8 * np.linalg.norm(xo), i
         true = np.linalg.norm(bs[i] - O.spmv_csr(A, xi)) / np.linalg.norm(bs[i])
         assert true <= 1.01e-12 and abs(true - rr[i]) <= 1e-14
+
+
+@pytest.mark.parametrize("bs", [1, 2, 8, 32, 5])
+@pytest.mark.parametrize("n", [37, 700, 4101, 9001, 30011, 80000])
+@pytest.mark.parametrize("name", ["cg", "bicgstab"])
+def test_block_jacobi_shapes(gko, name, n, bs):
+    """Block-Jacobi in the single-launch solvers (sizes that leave a short last
+    block; block size 5 takes the multi-kernel solve), FP64 and mixed."""
+    G = gko
+    A = banded_system(n, 7, name == "cg", n)
+    M = G.from_csr(A)
+    bj = dict(preconditioner=G.PRECOND_BLOCK_JACOBI, block_size=bs)
+    check(G, name, A, M, **bj)
+    check(G, name, A, M, precision=G.PRECISION_MIXED_F32, **bj)
