@@ -1,6 +1,6 @@
 // Host side of the single-launch solvers (persist.cuh): which systems they
 // take, the launch shape and the workspace.
-#include "persist.cuh"
+#include "persist_gmres.cuh"
 
 namespace gko {
 
@@ -16,6 +16,12 @@ template <>
 PkKernel<float, float> pk_bicg<float, float>(int, bool);
 template <>
 PkKernel<float, __nv_bfloat16> pk_bicg<float, __nv_bfloat16>(int, bool);
+template <>
+PkGmresKernel<double, double> pk_gmres<double, double>(int, bool);
+template <>
+PkGmresKernel<float, float> pk_gmres<float, float>(int, bool);
+template <>
+PkGmresKernel<float, __nv_bfloat16> pk_gmres<float, __nv_bfloat16>(int, bool);
 
 namespace {
 
@@ -25,6 +31,53 @@ const Buf& cols_of(const gko_matrix_s* A) {
 }
 const Buf& vals_of(const gko_matrix_s* A) {
   return A->fmt == GKO_CSR ? A->val : A->fmt == GKO_ELL ? A->ell_val : A->sellp_val;
+}
+
+// What every kernel is given: the matrix, right-hand side, x and options.
+template <typename T, typename VT>
+PkArgs<T, VT> args_of(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSpec& sp, size_t K) {
+  PkArgs<T, VT> a{};
+  a.n = (int32_t)A->n_rows;
+  a.K = (int32_t)K;
+  a.fmt = A->fmt;
+  a.rp = A->fmt == GKO_CSR ? ptr<int32_t>(A->row_ptr) : A->fmt == GKO_SELLP ? ptr<int32_t>(A->sellp_sets) : nullptr;
+  a.col = ptr<int32_t>(cols_of(A));
+  a.val = ptr<VT>(vals_of(A));
+  a.stride = A->stride;
+  a.slice = A->slice;
+  a.b = b;
+  a.x = x;
+  a.d = static_cast<const T*>(sp.minv);
+  a.bj = static_cast<const T*>(sp.bj);
+  a.bs = sp.bs;
+  a.rel_tol = sp.rel_tol;
+  a.maxit = sp.maxit;
+  a.check_true = sp.check_true;
+  a.x_zero = x_zero ? 1 : 0;
+  if (sp.rel) {
+    a.val64 = ptr<double>(vals_of(sp.rel->A64));
+    a.b64 = sp.rel->b64;
+    a.x64 = sp.rel->x64;
+    a.delta = sp.rel->delta;
+  }
+  a.err = device_error_word();
+  return a;
+}
+
+// Waits for the solve and reads its result.
+template <typename T>
+int finish(const Ctl* c, cudaStream_t s, SolveOut* out) {
+  Ctl* hc = host_ctl();
+  GKO_TRY(read_ctl(c, hc, s));
+  if (hc->half) return fail(GKO_TIMEOUT, "single-launch solve: a grid reduction's wait timed out");
+  out->status = hc->status;
+  out->iterations = hc->iter;
+  out->cycles = hc->cycles;
+  if (sizeof(T) == 8) {
+    out->have_residual = true;
+    out->rel_residual = hc->nb == 0.0 ? 0.0 : sqrt(hc->rr) / hc->nb;
+  }
+  return GKO_OK;
 }
 
 template <typename T, typename VT>
@@ -69,34 +122,10 @@ int launch(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const Solv
   Scratch mem;
   GKO_TRY(mem.get(sizeof(Ctl) + slot_bytes + 1024 + (size_t)nvec * (sizeof(T) * (size_t)n + 320), s));
   Carve cv{static_cast<char*>(mem.data())};
-  PkArgs<T, VT> a{};
-  a.n = (int32_t)n;
-  a.K = (int32_t)K;
-  a.fmt = A->fmt;
-  a.rp = A->fmt == GKO_CSR ? ptr<int32_t>(A->row_ptr) : A->fmt == GKO_SELLP ? ptr<int32_t>(A->sellp_sets) : nullptr;
-  a.col = ptr<int32_t>(cols_of(A));
-  a.val = ptr<VT>(vals_of(A));
-  a.stride = A->stride;
-  a.slice = A->slice;
-  a.b = b;
-  a.x = x;
-  a.d = static_cast<const T*>(sp.minv);
-  a.bj = static_cast<const T*>(sp.bj);
-  a.bs = sp.bs;
-  a.rel_tol = sp.rel_tol;
-  a.maxit = sp.maxit;
-  a.check_true = sp.check_true;
-  a.x_zero = x_zero ? 1 : 0;
-  if (sp.rel) {
-    a.val64 = ptr<double>(vals_of(sp.rel->A64));
-    a.b64 = sp.rel->b64;
-    a.x64 = sp.rel->x64;
-    a.delta = sp.rel->delta;
-  }
+  PkArgs<T, VT> a = args_of<T, VT>(A, b, x, x_zero, sp, K);
   a.c = cv.take<Ctl>(1);
   if (!cluster) a.slots = cv.take<ulonglong2>(2 * kPkMaxBlocks * kPkSlot);
   for (int k = 0; k < nvec; ++k) a.vec[k] = cv.take<T>((size_t)n);
-  a.err = device_error_word();
   if (!cluster) GKO_TRY_CUDA(cudaMemsetAsync(a.slots, 0, slot_bytes, s));
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // the blocks cannot all be resident
@@ -104,17 +133,7 @@ int launch(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const Solv
     return GKO_NOT_SUPPORTED;
   }
   GKO_TRY_CUDA(e);
-  Ctl* hc = host_ctl();
-  GKO_TRY(read_ctl(a.c, hc, s));
-  if (hc->half) return fail(GKO_TIMEOUT, "single-launch solve: a grid reduction's wait timed out");
-  out->status = hc->status;
-  out->iterations = hc->iter;
-  out->cycles = hc->cycles;
-  if (sizeof(T) == 8) {
-    out->have_residual = true;
-    out->rel_residual = hc->nb == 0.0 ? 0.0 : sqrt(hc->rr) / hc->nb;
-  }
-  return GKO_OK;
+  return finish<T>(a.c, s, out);
 }
 
 template <typename T, typename VT>
@@ -153,13 +172,58 @@ int run(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSp
   return GKO_NOT_SUPPORTED;
 }
 
+// GMRES: grid shapes only; the smallest that covers n with one block per SM.
+template <typename T, typename VT>
+int run_gmres(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSpec& sp, cudaStream_t s,
+              SolveOut* out) {
+  const int64_t n = A->n_rows;
+  const size_t K = (size_t)std::max<int32_t>(1, A->fmt == GKO_CSR ? A->plan.max_len : A->K);
+  for (bool staged : {true, false})
+    for (int shape : {11, 12, 13, 14, 9, 10}) {
+      const PkShape h = kPkShapes[shape];
+      const int64_t rb = (int64_t)h.nt * h.rpt, G = (n + rb - 1) / rb;
+      const size_t smem = staged ? K * (size_t)rb * (sizeof(VT) + sizeof(int32_t)) : 0;
+      const PkGmresKernel<T, VT> kern = pk_gmres<T, VT>(shape, staged);
+      if (!kern || G > std::min(sm_count(), kPkMaxBlocks) || smem > kPkSmemMax) continue;
+      if (smem > 24 * 1024)
+        GKO_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPkSmemMax));
+      const int64_t ld = (n + 63) / 64 * 64;
+      const size_t words = 2 * kPkMaxBlocks * kPkSlot + 2 * 32 * kPkMaxBlocks + 2 * 32 * 2;
+      Scratch mem;
+      GKO_TRY(mem.get(sizeof(Ctl) + sizeof(ulonglong2) * words + 2048 + sizeof(T) * ((size_t)n + (size_t)ld * (sp.restart + 1)),
+                      s));
+      Carve cv{static_cast<char*>(mem.data())};
+      PkGmresArgs<T, VT> g{};
+      g.a = args_of<T, VT>(A, b, x, x_zero, sp, K);
+      g.a.c = cv.take<Ctl>(1);
+      g.a.slots = cv.take<ulonglong2>(words);
+      g.sums = g.a.slots + 2 * kPkMaxBlocks * kPkSlot;
+      g.totals = g.sums + 2 * 32 * kPkMaxBlocks;
+      g.a.vec[0] = cv.take<T>((size_t)n);
+      g.V = cv.take<T>((size_t)ld * (sp.restart + 1));
+      g.ld = ld;
+      g.m = sp.restart;
+      GKO_TRY_CUDA(cudaMemsetAsync(g.a.slots, 0, sizeof(ulonglong2) * words, s));
+      void* args[] = {&g};
+      const cudaError_t e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)G), dim3((unsigned)h.nt), args,
+                                                        smem, s);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {  // the blocks cannot all be resident
+        cudaGetLastError();
+        continue;
+      }
+      GKO_TRY_CUDA(e);
+      return finish<T>(g.a.c, s, out);
+    }
+  return GKO_NOT_SUPPORTED;
+}
+
 }  // namespace
 
 int persist_solve(const gko_matrix_s* A, const double* b, void* x, bool x_zero, const SolveSpec& sp, cudaStream_t s,
                   SolveOut* out) {
   // CSR under the row-block plan (regular rows: other plans keep their SpMV
   // kernels), ELL and SELL-P; reliable updates for BiCGSTAB only
-  if (sp.solver > 1 || A->n_rows <= 0 || A->n_rows > kSmallRows) return GKO_NOT_SUPPORTED;
+  if (A->n_rows <= 0 || A->n_rows > kSmallRows) return GKO_NOT_SUPPORTED;
   if (sp.bj && (sp.bs & (sp.bs - 1))) return GKO_NOT_SUPPORTED;  // diagonal blocks end with thread blocks
   if (!(A->fmt == GKO_CSR && A->plan.kind == 1) && A->fmt != GKO_ELL && A->fmt != GKO_SELLP) return GKO_NOT_SUPPORTED;
   if (sp.rel && (sp.solver != 1 || sp.rel->A64->fmt != A->fmt)) return GKO_NOT_SUPPORTED;
@@ -170,12 +234,17 @@ int persist_solve(const gko_matrix_s* A, const double* b, void* x, bool x_zero, 
     return GKO_NOT_SUPPORTED;
   }
   if (!coop) return GKO_NOT_SUPPORTED;
+  const bool gmres = sp.solver == 2;
+  if (gmres && sp.restart > kPkRestart) return GKO_NOT_SUPPORTED;
   switch (A->dtype) {
     case GKO_F64:
+      if (gmres) return run_gmres<double, double>(A, b, static_cast<double*>(x), x_zero, sp, s, out);
       return run<double, double>(A, b, static_cast<double*>(x), x_zero, sp, s, out);
     case GKO_F32:
+      if (gmres) return run_gmres<float, float>(A, b, static_cast<float*>(x), x_zero, sp, s, out);
       return run<float, float>(A, b, static_cast<float*>(x), x_zero, sp, s, out);
     case GKO_BF16:
+      if (gmres) return run_gmres<float, __nv_bfloat16>(A, b, static_cast<float*>(x), x_zero, sp, s, out);
       return run<float, __nv_bfloat16>(A, b, static_cast<float*>(x), x_zero, sp, s, out);
   }
   return GKO_NOT_SUPPORTED;

@@ -159,3 +159,32 @@ def test_block_jacobi_shapes(gko, name, n, bs):
     bj = dict(preconditioner=G.PRECOND_BLOCK_JACOBI, block_size=bs)
     check(G, name, A, M, **bj)
     check(G, name, A, M, precision=G.PRECISION_MIXED_F32, **bj)
+
+
+@pytest.mark.parametrize("restart", [1, 7, 30, 31, 32])
+@pytest.mark.parametrize("n", [1, 33, 700, 9001, 40000, 77825, 200000])
+def test_gmres_shapes_and_restarts(gko, n, restart):
+    """The single-launch GMRES over its launch shapes and restart lengths (32
+    takes the multi-kernel solve): the oracle's solution at 1e-12, the true
+    residual reported, repeatable, and capped in the middle of a cycle."""
+    G = gko
+    A = banded_system(n, 7, False, n)
+    M = G.from_csr(A)
+    b = np.random.default_rng(1).uniform(-1, 1, n)
+    for opt in ({}, {"precision": G.PRECISION_MIXED_F32}):
+        xd = dev(np.zeros(n))
+        res = G.gko_solve_gmres(M, dev(b), xd, 1e-12, 3000, G.opts(restart=restart, **opt))
+        x = host(xd)
+        xo, ro = O.gmres(A, b, tol=1e-12, maxit=3000, restart=restart)
+        assert res.status == G.OK and ro.status == 0, res
+        assert np.linalg.norm(x - xo) <= 1e-8 * np.linalg.norm(xo)
+        true = np.linalg.norm(b - O.spmv_csr(A, x)) / np.linalg.norm(b)
+        assert true <= 1.01e-12 and abs(true - res.rel_residual) <= 1e-13
+        xd2 = dev(np.zeros(n))
+        G.gko_solve_gmres(M, dev(b), xd2, 1e-12, 3000, G.opts(restart=restart, **opt))
+        assert host(xd2).tobytes() == x.tobytes()
+    xd = dev(np.zeros(n))
+    res = G.gko_solve_gmres(M, dev(b), xd, 1e-15, 2, G.opts(restart=restart))
+    assert res.iterations <= 2
+    true = np.linalg.norm(b - O.spmv_csr(A, host(xd))) / np.linalg.norm(b)
+    assert abs(true - res.rel_residual) <= 1e-13
