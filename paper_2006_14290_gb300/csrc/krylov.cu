@@ -864,31 +864,89 @@ __global__ void __launch_bounds__(256, 4) gm_scale_kernel(int64_t n, T* __restri
   GKO_GRID_LOOP(i, n) v[i] = sc.scale(v[i]);
 }
 
-// gated multi-dot: partial sums of V_j . w for j <= jmax (blockIdx.y = j)
-template <typename T>
-__global__ void __launch_bounds__(256, 4) gm_multidot_kernel(int64_t n, const T* __restrict__ V, int64_t ldv,
-                                                          const T* __restrict__ w, double* __restrict__ partials,
-                                                          Ctl* c, int pass) {
-  pdl_begin();
-  if (gated(&c->phase) || (pass == 1 && *(volatile int*)&c->noreorth)) return;
-  const int j = blockIdx.y;
-  const T* v = V + (int64_t)j * ldv;
-  double acc = 0.0;
-  GKO_GRID_LOOP(i, n) acc = __fma_rn(wd(v[i]), wd(__ldg(w + i)), acc);
-  const double sblk = block_sum<256>(acc);
-  if (threadIdx.x == 0) partials[(int64_t)j * kMultiSlots + blockIdx.x] = sblk;
+// h_j = V_j . w for the k basis vectors in groups of up to kDotGroup: a block
+// takes one group over a chunk of the rows, so that a load of w serves four
+// products, and the group's last block adds the chunks' sums.  A group of J
+// vectors gets J / k of the blocks: every block has the same work (equal
+// chunks left the last blocks running alone, 75 us instead of 63 for 13
+// vectors).  The FP64 pipe bounds it (one FMA per 8 bytes of V: 0.53 T FMA/s,
+// 4.2 TB/s).
+constexpr int kMaxRestart = 128, kDotGroup = 4, kMaxDotGroups = kMaxRestart / kDotGroup;
+
+template <typename T, int J>
+__device__ __forceinline__ void dot_group(int64_t n, const T* V, int64_t ldv, const T* w, int64_t tid, int64_t nth,
+                                          double (&acc)[kDotGroup]) {
+  constexpr int VN = Vec16<T>::N;
+  const int64_t nv = n / VN;
+  for (int64_t iv = tid; iv < nv; iv += nth) {
+    const Vec16<T> ww = vload(w + iv * VN);
+    Vec16<T> v[J];
+#pragma unroll
+    for (int q = 0; q < J; ++q) v[q] = vload(V + q * ldv + iv * VN);
+#pragma unroll
+    for (int e = 0; e < VN; ++e) {
+      const double we = wd(ww.v[e]);
+#pragma unroll
+      for (int q = 0; q < J; ++q) acc[q] = __fma_rn(wd(v[q].v[e]), we, acc[q]);
+    }
+  }
+  if (const int64_t r = nv * VN + tid; r < n) {
+    const double we = wd(w[r]);
+#pragma unroll
+    for (int q = 0; q < J; ++q) acc[q] = __fma_rn(wd(V[q * ldv + r]), we, acc[q]);
+  }
 }
 
-__global__ void __launch_bounds__(256, 4) gm_multidot_finish_kernel(int g, const double* __restrict__ partials,
-                                                                 double* __restrict__ h, int accumulate, Ctl* c,
-                                                                 int pass) {
+template <typename T>
+__global__ void __launch_bounds__(256, 4) gm_multidot_kernel(int64_t n, int k, const T* __restrict__ V, int64_t ldv,
+                                                          const T* __restrict__ w, double* __restrict__ h,
+                                                          double* partials, unsigned* counters, Ctl* c, int pass) {
+  __shared__ int is_last;
   pdl_begin();
   if (gated(&c->phase) || (pass == 1 && *(volatile int*)&c->noreorth)) return;
-  const int j = blockIdx.x;
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < g; i += 256) acc += partials[(int64_t)j * kMultiSlots + i];
-  const double t = block_sum<256>(acc);
-  if (threadIdx.x == 0) h[j] = accumulate ? h[j] + t : t;
+  // group y: vectors j0 .. j0 + J - 1 and the blocks first .. first + chunks - 1
+  // (gridDim.x >= k: a block or more for each vector)
+  const int groups = (k + kDotGroup - 1) / kDotGroup, G = gridDim.x, B = blockIdx.x;
+  int y = 0, j0 = 0, first = 0, J = 0, chunks = 0;
+  for (;; ++y) {
+    j0 = y * k / groups;
+    const int j1 = (y + 1) * k / groups;
+    first = (int)((int64_t)j0 * G / k);
+    J = j1 - j0;
+    chunks = (int)((int64_t)j1 * G / k) - first;
+    if (B < first + chunks) break;
+  }
+  const T* v = V + (int64_t)j0 * ldv;
+  const int64_t tid = (int64_t)(B - first) * 256 + threadIdx.x, nth = (int64_t)chunks * 256;
+  double acc[kDotGroup] = {};
+  switch (J) {
+    case 1: dot_group<T, 1>(n, v, ldv, w, tid, nth, acc); break;
+    case 2: dot_group<T, 2>(n, v, ldv, w, tid, nth, acc); break;
+    case 3: dot_group<T, 3>(n, v, ldv, w, tid, nth, acc); break;
+    default: dot_group<T, 4>(n, v, ldv, w, tid, nth, acc); break;
+  }
+  block_sum_n<256, kDotGroup>(acc);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int q = 0; q < kDotGroup; ++q) partials[(int64_t)q * G + B] = acc[q];
+    __threadfence();
+    is_last = atomicAdd(counters + y, 1u) == (unsigned)chunks - 1u;
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+#pragma unroll
+  for (int q = 0; q < kDotGroup; ++q) {
+    acc[q] = 0.0;
+    for (int i = threadIdx.x; i < chunks; i += 256) acc[q] += __ldcg(partials + (int64_t)q * G + first + i);
+  }
+  block_sum_n<256, kDotGroup>(acc);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int q = 0; q < kDotGroup; ++q)
+      if (q < J) h[j0 + q] = acc[q];
+    counters[y] = 0u;
+  }
 }
 
 struct StoreRr {
@@ -902,7 +960,6 @@ struct StoreRr {
 
 // w -= sum_{j<=jmax} h_j V_j (h: device, the pass's coefficients); with
 // NORM also reduces ||w||^2 into c->rr.
-constexpr int kMaxRestart = 128;
 
 // -h_j as the coefficient pair of Lin<T>, built once per block
 template <typename T>
@@ -927,6 +984,29 @@ __device__ __forceinline__ T lin_apply(T hi, T lo, T x, T y) {
   else return __fma_rn(hi, x, y);
 }
 
+// v_e -= ... over the columns 0 .. k-1 for VN rows at a time; four columns'
+// loads in flight
+template <typename T>
+__device__ __forceinline__ void axpy_cols(int k, const T* s_hi, const T* s_lo, const T* V, int64_t ldv, int64_t i0,
+                                          Vec16<T>& v) {
+  constexpr int U = 4;
+  int j = 0;
+  for (; j + U <= k; j += U) {
+    Vec16<T> u[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) u[q] = vload(V + (j + q) * ldv + i0);
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+#pragma unroll
+      for (int e = 0; e < Vec16<T>::N; ++e) v.v[e] = lin_apply<T>(s_hi[j + q], s_lo[j + q], u[q].v[e], v.v[e]);
+  }
+  for (; j < k; ++j) {
+    const Vec16<T> u = vload(V + j * ldv + i0);
+#pragma unroll
+    for (int e = 0; e < Vec16<T>::N; ++e) v.v[e] = lin_apply<T>(s_hi[j], s_lo[j], u.v[e], v.v[e]);
+  }
+}
+
 template <typename T, bool NORM>
 __global__ void __launch_bounds__(256, 4) gm_axpy_kernel(int64_t n, int jcount, const double* __restrict__ h,
                                                       const T* __restrict__ V, int64_t ldv, T* __restrict__ w, Ctl* c,
@@ -935,8 +1015,21 @@ __global__ void __launch_bounds__(256, 4) gm_axpy_kernel(int64_t n, int jcount, 
   __shared__ T s_hi[kMaxRestart + 1], s_lo[kMaxRestart + 1];
   if (gated(&c->phase) || (pass == 1 && *(volatile int*)&c->noreorth)) return;
   load_coefs<T>(h, jcount, -1.0, s_hi, s_lo);
+  constexpr int VN = Vec16<T>::N;
   double acc[1] = {0.0};
-  GKO_GRID_LOOP(i, n) {
+  const int64_t nv = n / VN;
+  GKO_GRID_LOOP(iv, nv) {
+    Vec16<T> v = vload(w + iv * VN);
+    axpy_cols(jcount, s_hi, s_lo, V, ldv, iv * VN, v);
+    vstore(w + iv * VN, v);
+    if (NORM)
+#pragma unroll
+      for (int e = 0; e < VN; ++e) {
+        const double ow = wd(v.v[e]);
+        acc[0] = __fma_rn(ow, ow, acc[0]);
+      }
+  }
+  if (const int64_t i = nv * VN + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n) {
     T v = w[i];
     for (int j = 0; j < jcount; ++j) v = lin_apply<T>(s_hi[j], s_lo[j], V[(int64_t)j * ldv + i], v);
     w[i] = v;
@@ -950,24 +1043,31 @@ __global__ void __launch_bounds__(256, 4) gm_axpy_kernel(int64_t n, int jcount, 
 
 // Column j of the Hessenberg matrix from the two CGS passes, previous Givens
 // rotations, a new rotation, the residual estimate |g_{j+1}| and the cycle
-// end test.  One thread.
-__global__ void gm_givens_kernel(int j, int m, const double* __restrict__ h1, const double* __restrict__ h2,
-                                 double* __restrict__ H, double* __restrict__ cs, double* __restrict__ sn,
-                                 double* __restrict__ g, Ctl* c) {
-  pdl_begin();
-  if (gated(&c->phase)) return;
-  double* col = H + (int64_t)j;  // H[i*m + j]
+// end test: thread 0, from shared memory (a chain of j rotations of two
+// dependent FP64 operations each; reading H from global memory as it went made
+// it 10 us at j = 15).
+__device__ __forceinline__ void gm_givens(int j, int m, const double* h1, const double* h2, double* H, double* cs,
+                                          double* sn, double* g, Ctl* c) {
+  __shared__ double s_h[kMaxRestart + 1], s_c[kMaxRestart], s_s[kMaxRestart];
   const bool two = !c->noreorth;
-  for (int i = 0; i <= j; ++i) col[(int64_t)i * m] = two ? h1[i] + h2[i] : h1[i];
-  const double hn = sqrt(c->rr);
-  col[(int64_t)(j + 1) * m] = hn;
-  for (int i = 0; i < j; ++i) {
-    const double a = col[(int64_t)i * m], b = col[(int64_t)(i + 1) * m];
-    col[(int64_t)i * m] = cs[i] * a + sn[i] * b;
-    col[(int64_t)(i + 1) * m] = -sn[i] * a + cs[i] * b;
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+    s_h[i] = two ? h1[i] + h2[i] : h1[i];
+    if (i < j) {
+      s_c[i] = cs[i];
+      s_s[i] = sn[i];
+    }
   }
-  const double a = col[(int64_t)j * m], b = col[(int64_t)(j + 1) * m];
-  const double den = sqrt(a * a + b * b);
+  __syncthreads();
+  if (threadIdx.x) return;
+  double* col = H + (int64_t)j;  // H[i*m + j]
+  const double hn = sqrt(c->rr);
+  double a = s_h[0];
+  for (int i = 0; i < j; ++i) {
+    const double b = s_h[i + 1];
+    col[(int64_t)i * m] = s_c[i] * a + s_s[i] * b;
+    a = -s_s[i] * a + s_c[i] * b;
+  }
+  const double den = sqrt(a * a + hn * hn);
   c->iter += 1;
   c->k = j + 1;
   if (den == 0.0) {
@@ -977,24 +1077,43 @@ __global__ void gm_givens_kernel(int j, int m, const double* __restrict__ h1, co
     return;
   }
   cs[j] = a / den;
-  sn[j] = b / den;
+  sn[j] = hn / den;
   col[(int64_t)j * m] = den;
-  col[(int64_t)(j + 1) * m] = 0.0;
   g[j + 1] = -sn[j] * g[j];
   g[j] = cs[j] * g[j];
-  c->rho = hn;  // h_{j+1,j}, the divisor of the next basis vector
   if (hn == 0.0 || fabs(g[j + 1]) <= c->tol_abs) c->replace = 1;  // estimate says converged
   if (c->replace || c->iter >= c->maxit || j + 1 == m) c->phase = 1;
 }
 
-// v_{j+1} = w / h_{j+1,j} (skipped once the cycle has ended)
+// v_{j+1} = w / h_{j+1,j}, and beside it, in the last block, the step's
+// scalars.  The division needs the norm alone, so neither waits for the other
+// (two launches of 10 us each before); after the cycle's last step v_{j+1} is
+// not read.
 template <typename T>
-__global__ void __launch_bounds__(256, 4) gm_next_kernel(int64_t n, const T* __restrict__ w, T* __restrict__ vn,
-                                                      Ctl* c) {
+__global__ void __launch_bounds__(256, 4) gm_next_kernel(int64_t n, const T* __restrict__ w, T* __restrict__ vn, int j,
+                                                      int m, const double* __restrict__ h1,
+                                                      const double* __restrict__ h2, double* __restrict__ H,
+                                                      double* __restrict__ cs, double* __restrict__ sn,
+                                                      double* __restrict__ g, Ctl* c) {
   pdl_begin();
-  if (gated(&c->phase)) return;
-  const Lin<T> sc = block_bcast<Lin<T>>([&] { return Lin<T>(1.0 / c->rho); });
-  GKO_GRID_LOOP(i, n) vn[i] = sc.scale(w[i]);
+  __shared__ int off;  // the last block may set the gate while others start
+  if (threadIdx.x == 0) off = gated(&c->phase);
+  __syncthreads();
+  if (off) return;
+  if (blockIdx.x == gridDim.x - 1) {
+    gm_givens(j, m, h1, h2, H, cs, sn, g, c);
+    return;
+  }
+  const Lin<T> sc = block_bcast<Lin<T>>([&] { return Lin<T>(1.0 / sqrt(c->rr)); });
+  constexpr int VN = Vec16<T>::N;
+  const int64_t nth = (int64_t)(gridDim.x - 1) * 256, tid = blockIdx.x * 256ll + threadIdx.x, nv = n / VN;
+  for (int64_t iv = tid; iv < nv; iv += nth) {
+    Vec16<T> v = vload(w + iv * VN);
+#pragma unroll
+    for (int e = 0; e < VN; ++e) v.v[e] = sc.scale(v.v[e]);
+    vstore(vn + iv * VN, v);
+  }
+  if (const int64_t i = nv * VN + tid; i < n) vn[i] = sc.scale(w[i]);
 }
 
 // Back substitution H[0:k,0:k] y = g[0:k]; stores -y for the x update.
@@ -1020,7 +1139,15 @@ __global__ void __launch_bounds__(256, 4) gm_update_x_kernel(int64_t n, const do
   if (gated(&c->done)) return;
   const int k = c->k;
   load_coefs<T>(ny, k, -1.0, s_hi, s_lo);
-  GKO_GRID_LOOP(i, n) {
+  constexpr int VN = Vec16<T>::N;
+  const int64_t nv = al16(x) ? n / VN : 0;
+  GKO_GRID_LOOP(iv, nv) {
+    Vec16<T> v = vload(x + iv * VN);
+    axpy_cols(k, s_hi, s_lo, V, ldv, iv * VN, v);
+    vstore(x + iv * VN, v);
+  }
+  for (int64_t i = nv * VN + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     T v = x[i];
     for (int j = 0; j < k; ++j) v = lin_apply<T>(s_hi[j], s_lo[j], V[(int64_t)j * ldv + i], v);
     x[i] = v;
@@ -1140,9 +1267,10 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
   const T* bj = static_cast<const T*>(sp.bj);  // block-Jacobi inverse blocks
   const int bs = sp.bs;
   const size_t spmv_sb = spmv_scratch_bytes(A);
+  const int slots = std::max(kMaxRestart, 4 * sm_count());  // partial sums of a multi-dot's group member
   const size_t bytes = 256 * 16 + sizeof(Ctl) + sizeof(double) * 3 * kDotSlots + 512 +
                        (size_t)nvec * (sizeof(T) * ((size_t)n + 64) + 320) + spmv_sb + 320 +
-                       sizeof(double) * ((size_t)(m + 1) * m + 6 * (m + 2) + (size_t)(m + 1) * kMultiSlots) + 4096;
+                       sizeof(double) * ((size_t)(m + 1) * m + 6 * (m + 2) + (size_t)kDotGroup * slots) + 4096;
   Scratch mem;
   GKO_TRY(mem.get(bytes, s));
   Carve cv{static_cast<char*>(mem.data())};
@@ -1340,7 +1468,9 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
     double* h1 = cv.take<double>(m + 2);
     double* h2 = cv.take<double>(m + 2);
     double* ny = cv.take<double>(m + 2);
-    double* mpart = cv.take<double>((size_t)(m + 1) * kMultiSlots);
+    double* mpart = cv.take<double>((size_t)kDotGroup * slots);
+    unsigned* dcount = cv.take<unsigned>(kMaxDotGroups);
+    GKO_TRY_CUDA(cudaMemsetAsync(dcount, 0, sizeof(unsigned) * kMaxDotGroups, s));
     // ||b|| and the zero-b case through the common init kernel
     init_residual_kernel<T><<<rg, 256, 0, s>>>(n, b, nullptr, w, nullptr, nullptr, nullptr, nullptr, ws,
                                                InitOp{c, sp.rel_tol, 2});
@@ -1357,7 +1487,6 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
       GKO_TRY_CUDA(cudaMemsetAsync(&c->status, 0, sizeof(int), s));
       hc->done = 0;
     }
-    int64_t mg = std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, kMultiSlots));
     bool first = true;
     while (!hc->done) {
       // cycle start: v0 = b - A x
@@ -1383,18 +1512,15 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
         // shrank ||w|| below ||w0|| / sqrt(2) (selective reorthogonalisation)
         for (int pass = 0; pass < 2; ++pass) {
           double* hp = pass == 0 ? h1 : h2;
-          GKO_TRY_CUDA(launch_k(gm_multidot_kernel<T>, dim3((unsigned)mg, (unsigned)(j + 1)), dim3(256), 0, s, n,
-                                (const T*)V, ld, (const T*)w, mpart, c, pass));
-          GKO_TRY_CUDA(launch_k(gm_multidot_finish_kernel, dim3(j + 1), dim3(256), 0, s, (int)mg,
-                                (const double*)mpart, hp, 0, c, pass));
+          // one wave of blocks, 1,024 rows of four vectors or more to a block
+          const int64_t blocks = std::max<int64_t>(j + 1, std::min<int64_t>((n + 4095) / 4096 * (j + 1), slots));
+          GKO_TRY_CUDA(launch_k(gm_multidot_kernel<T>, dim3((unsigned)blocks), dim3(256), 0, s, n,
+                                j + 1, (const T*)V, ld, (const T*)w, hp, mpart, dcount, c, pass));
           GKO_TRY_CUDA(launch_k(gm_axpy_kernel<T, true>, dim3(rg), dim3(256), 0, s, n, j + 1, (const double*)hp,
                                 (const T*)V, ld, w, c, ws, pass));
         }
-        GKO_TRY_CUDA(launch_k(gm_givens_kernel, dim3(1), dim3(1), 0, s, j, m, (const double*)h1, (const double*)h2, H,
-                              cs, sn, g, c));
-        if (j + 1 <= m)
-          GKO_TRY_CUDA(launch_k(gm_next_kernel<T>, dim3(vg), dim3(256), 0, s, n, (const T*)w,
-                                V + (int64_t)(j + 1) * ld, c));
+        GKO_TRY_CUDA(launch_k(gm_next_kernel<T>, dim3(vg + 1), dim3(256), 0, s, n, (const T*)w,
+                              V + (int64_t)(j + 1) * ld, j, m, (const double*)h1, (const double*)h2, H, cs, sn, g, c));
       }
       gm_backsolve_kernel<<<1, 1, 0, s>>>(m, H, g, ny, c);
       gm_update_x_kernel<T><<<vg, 256, 0, s>>>(n, ny, V, ld, x, c);

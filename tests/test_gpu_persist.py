@@ -161,11 +161,11 @@ def test_block_jacobi_shapes(gko, name, n, bs):
     check(G, name, A, M, precision=G.PRECISION_MIXED_F32, **bj)
 
 
-@pytest.mark.parametrize("restart", [1, 7, 30, 31, 32])
+@pytest.mark.parametrize("restart", [1, 7, 30, 31, 32, 128])
 @pytest.mark.parametrize("n", [1, 33, 700, 9001, 40000, 77825, 200000])
 def test_gmres_shapes_and_restarts(gko, n, restart):
-    """The single-launch GMRES over its launch shapes and restart lengths (32
-    takes the multi-kernel solve): the oracle's solution at 1e-12, the true
+    """The single-launch GMRES over its launch shapes and restart lengths (32 and 128
+    take the multi-kernel solve): the oracle's solution at 1e-12, the true
     residual reported, repeatable, and capped in the middle of a cycle."""
     G = gko
     A = banded_system(n, 7, False, n)
