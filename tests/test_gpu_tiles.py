@@ -54,3 +54,34 @@ def test_tiles_match_oracle(gko, name, A, fmt, dt):
             G.gko_spmv(alpha, M, dev(x32), beta, yd)
             check_spmv_f32(host(yd), A, x32.astype(np.float64), alpha, beta, y0.astype(np.float32).astype(np.float64),
                            v if dt == "f32" else bf16_round(A.val))
+
+
+@pytest.mark.parametrize("S", [2, 4])
+@pytest.mark.parametrize("extra", [0, 1, 64])
+@pytest.mark.parametrize("waves", [0, 1, 2, 3, 5])
+def test_deferred_row_sums(gko, S, extra, waves):
+    """FP64 row-block CSR with S lanes a row keeps the sums of up to S row
+    blocks before it reduces them: 0 to 5 row blocks per thread block and a
+    ragged last one, plain, with alpha and beta, and with the fused dot."""
+    G = gko
+    n = max(1, waves * 152 * 9 * (128 // S) + extra)
+    rng = np.random.default_rng(n)
+    lens = rng.integers(0, 12, n)
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    row = np.repeat(np.arange(n), lens)
+    col = (row + rng.integers(0, 40, row.size)) % n
+    A = I.Csr(n, n, rp, col.astype(np.int32), rng.uniform(-1, 1, row.size), "rows of 0..11")
+    M = G.from_csr(A)
+    M.set_plan(1, S, 1, 1024)
+    x, y = rng.uniform(-1, 1, n), rng.uniform(-1, 1, n)
+    yo = np.bincount(row, A.val * x[col], n)
+    bound = 2.0**-53 * (14 * np.bincount(row, np.abs(A.val * x[col]), n) + 1e-300)
+    yd = dev(y)
+    G.gko_spmv(1.0, M, dev(x), 0.0, yd)
+    assert np.all(np.abs(host(yd) - yo) <= bound)
+    yd = dev(y)
+    G.gko_spmv(-1.5, M, dev(x), 0.5, yd)
+    assert np.all(np.abs(host(yd) - (-1.5 * yo + 0.5 * y)) <= 2 * bound + 2.0**-52 * np.abs(y))
+    yd = dev(np.zeros(n))
+    d = G.gko_spmv_dot(M, dev(x), yd)  # x . (A x)
+    assert abs(d - x @ yo) <= 1e-13 * (np.abs(x) @ np.abs(yo)) + np.abs(x) @ bound
