@@ -80,6 +80,9 @@ int finish(const Ctl* c, cudaStream_t s, SolveOut* out) {
   return GKO_OK;
 }
 
+// Static shared memory of a CG or BiCGSTAB kernel, at most.
+constexpr size_t kPkStaticMax = sizeof(PkShared<512, kPkCluster>) + 1024;
+
 template <typename T, typename VT>
 int launch(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSpec& sp, cudaStream_t s, SolveOut* out,
            int shape, bool staged, int G, size_t K, size_t smem) {
@@ -88,9 +91,10 @@ int launch(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const Solv
   const bool cluster = sh.mode == kPkCluster;
   const PkKernel<T, VT> kern = sp.solver == 0 ? pk_cg<T, VT>(shape, staged) : pk_bicg<T, VT>(shape, staged);
   if (!kern) return GKO_NOT_SUPPORTED;
-  // always the largest request, so that concurrent solves (serving threads)
-  // never lower each other's limit
-  if (smem > 48 * 1024)
+  // The default limit of 48 KB holds static and dynamic shared memory together.
+  // Always the largest request, so that concurrent solves (serving threads)
+  // never lower each other's limit.
+  if (smem > 48 * 1024 - kPkStaticMax)
     GKO_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPkSmemMax));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)G);

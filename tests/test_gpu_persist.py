@@ -2,6 +2,10 @@
 (blocks of 32-512 rows in one cluster, then one block per SM) against the
 oracle: both sides to 1e-12, solutions within 1e-8 (kappa * 1e-12 << 1e-8),
 the reported residual the true one, as tests/test_gpu_solvers.py."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -10,6 +14,7 @@ from gpu_util import dev, host
 from paper_2006_14290_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def banded_system(n, half, spd, seed):
@@ -188,3 +193,41 @@ def test_gmres_shapes_and_restarts(gko, n, restart):
     assert res.iterations <= 2
     true = np.linalg.norm(b - O.spmv_csr(A, host(xd))) / np.linalg.norm(b)
     assert abs(true - res.rel_residual) <= 1e-13
+
+
+FRESH = """
+import sys, numpy as np, torch
+sys.path.insert(0, {root!r}); sys.path.insert(0, {root!r} + '/tests')
+from gpu_util import dev, host
+from paper_2006_14290_gb300 import gko as G, inputs as I
+def rows_of(K, n):
+    cols = np.arange(n)[:, None] + np.arange(-(K // 2), K - K // 2)[None, :]
+    vals = np.full(cols.shape, -1.0); vals[:, K // 2] = K + 1.0
+    ok = (cols >= 0) & (cols < n)
+    rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+    return G.from_csr(I.Csr(n, n, rp, cols[ok].astype(np.int32), vals[ok], 'rows'))
+def solve(K, n, opt):
+    xd = dev(np.zeros(n))
+    res = G.gko_solve_bicgstab(rows_of(K, n), dev(np.linspace(1, 2, n)), xd, 1e-12, 500, G.opts(**opt))
+    assert res.status == G.OK, res
+    return host(xd).tobytes()
+opt = {opt}
+first = solve({K}, {n}, opt)
+solve({K} + 2, {n}, opt)  # more shared memory: raises the kernel's limit
+assert solve({K}, {n}, opt) == first
+"""
+
+
+# entries (and published vectors) of 46 to 48 KB a block: 12 bytes an entry in FP64, 8 in FP32
+@pytest.mark.parametrize("K,n,opt", [(8, 40000, {}), (4, 80000, {}), (6, 8000, {}),
+                                     (12, 40000, {"precision": 1}), (6, 80000, {"precision": 1}),
+                                     (5, 8000, {"preconditioner": 2, "block_size": 8})])
+def test_shared_memory_just_below_the_default_limit(gko, K, n, opt):
+    """The same solve, bit for bit, before and after a larger one has raised
+    the kernel's shared-memory limit (in a process of its own: the limit stays
+    raised once any solve has done it)."""
+    G = gko
+    assert G.PRECISION_MIXED_F32 == 1 and G.PRECOND_BLOCK_JACOBI == 2
+    code = FRESH.format(root=ROOT, K=K, n=n, opt=opt)
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
