@@ -179,13 +179,18 @@ __global__ void __launch_bounds__(256, 4) init_residual_kernel(int64_t n, const 
   reduce_op<3>(acc, ws, op);
 }
 
-// t = b - q stored into q; ||t||^2 decides: converged, or replace r by t.
-// t[0] = ||t||^2, t[1] = t.(d t) (= t[0] without a preconditioner)
+// t = b - q stored into q; ||t||^2 decides: converged, out of iterations, or
+// replace r by t (close to the attainable accuracy the recurrence may meet the
+// tolerance in every step and the true residual in none, so the cap is tested
+// here too).  t[0] = ||t||^2, t[1] = t.(d t) (= t[0] without a preconditioner)
 struct TrueResOp {
   Ctl* c;
   __device__ void operator()(const double (&t)[2]) const {
     if (sqrt(t[0]) <= c->tol_abs) {
       c->status = kConverged;
+      c->done = 1;
+    } else if (c->iter >= c->maxit) {
+      c->status = kNotConverged;
       c->done = 1;
     } else {
       c->status = kRun;

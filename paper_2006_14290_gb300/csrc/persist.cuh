@@ -660,7 +660,9 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
       T tj[RPT];
       if (!true_residual(tj, [&](const double (&t)[2], double* o) {
             rr_true = t[0];
-            o[0] = sqrt(t[0]) <= tol ? 1.0 : 0.0;
+            // 0 go on, 1 converged, 3 iteration cap (close to the attainable accuracy the
+            // recurrence may meet the tolerance in every step and the true residual in none)
+            o[0] = sqrt(t[0]) <= tol ? 1.0 : it >= a.maxit ? 3.0 : 0.0;
             o[1] = pk_pack<T>(t[1] / rho_prev);
             rho = t[1];
           })) {
@@ -668,7 +670,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
         break;
       }
       if (pk_flag(sh.out[0])) {
-        status = kConverged;
+        status = sh.out[0] == 1.0 ? kConverged : kNotConverged;
         known = true;
         break;
       }

@@ -231,3 +231,24 @@ def test_shared_memory_just_below_the_default_limit(gko, K, n, opt):
     code = FRESH.format(root=ROOT, K=K, n=n, opt=opt)
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("precond", [0, 1, 2])
+@pytest.mark.parametrize("n,fmt", [(33, "csr"), (300, "csr"), (300, "ell"), (20000, "csr"), (300, "coo")])
+@pytest.mark.parametrize("name", ["cg", "bicgstab"])
+def test_iteration_cap_near_attainable_accuracy(gko, name, n, fmt, precond):
+    """A tolerance below what FP64 can reach: the recurrence residual meets it
+    again and again, the true residual never, and max_iters still ends the
+    solve wherever it falls (COO: the multi-kernel solve)."""
+    G = gko
+    if precond == 2 and fmt != "csr":
+        pytest.skip("block-Jacobi reads a CSR matrix")
+    A = banded_system(n, 7, name == "cg", 5)
+    M = G.from_csr(A)
+    M = {"csr": lambda m: m, "ell": G.gko_matrix_convert_to_ell, "coo": G.gko_matrix_convert_to_coo}[fmt](M)
+    b = np.random.default_rng(5).uniform(-1, 1, n)
+    for cap in range(1, 140 if n <= 300 and fmt != "coo" else 90):
+        x, res = solve(G, name, M, b, tol=1e-17, maxit=cap, preconditioner=precond)
+        assert res.iterations <= cap and res.status in (G.NOT_CONVERGED, G.BREAKDOWN), (cap, res)
+        true = np.linalg.norm(b - O.spmv_csr(A, x)) / np.linalg.norm(b)
+        assert abs(true - res.rel_residual) <= 1e-13
