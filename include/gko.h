@@ -599,6 +599,18 @@ GKO_API int gko_bench_gather(gko_dtype dtype, int32_t inner_loops, const void *x
  * Synchronises `stream`; the context stays usable. */
 GKO_API int gko_diag_bounded_wait(int64_t cycles, int32_t *timed_out, void *stream);
 
+/* Check and clock of the exchanges of the single-launch solvers (no
+ * counterpart in the paper): one cluster of 2..16 blocks, or a cooperative
+ * grid of 2 blocks up to one per SM, passes `steps` (1..1,000,000) steps that
+ * each add `values` (1..3) numbers per thread over all blocks, or (0) publish
+ * a vector, read a neighbour's part of it and pass a second barrier.
+ * out[3 b .. 3 b + 2] (host): block b's steps, its wrong totals and vector
+ * entries, and its slot words that do not carry the tag of their slot's last
+ * step; the latter two must be 0.  *cycles_per_step: SM clock cycles of block
+ * 0.  Synchronises `stream`; GKO_INVALID_ARG on sizes out of range. */
+GKO_API int gko_diag_exchange(int32_t cluster, int32_t blocks, int32_t values, int32_t steps, int32_t *out,
+                              double *cycles_per_step, void *stream);
+
 #ifdef __cplusplus
 }
 #endif

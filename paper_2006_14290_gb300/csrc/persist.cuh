@@ -84,9 +84,13 @@ struct PkArgs {
 // ----------------------------------------------------------- reduction --
 
 // A partial sum in flight: its low and its high 32 bits, each in an 8-byte
-// word with the exponent and the step's tag (16 bits: a slot's previous
-// contents are from two steps before).  The words are stored and loaded
-// whole, so a reader that sees both tags has the value.
+// word with the exponent and the step's tag.  The words are stored and loaded
+// whole, so a reader that sees both tags has the value.  16 bits of tag are
+// enough because every step stores all kPkWords words of a slot, used or not:
+// whatever a word held before is from two steps ago (were unused words left
+// alone, one could keep a tag that the same step number mod 65,536 matches
+// much later).
+constexpr int kPkWords = 3;
 __device__ __forceinline__ ulonglong2 pk_word(const Fx& f, unsigned tag) {
   const unsigned long long meta = (unsigned long long)((tag << 16) | ((unsigned)f.e & 0xffffu)) << 32;
   return make_ulonglong2(meta | (unsigned)f.v, meta | (unsigned)((unsigned long long)f.v >> 32));
@@ -140,7 +144,7 @@ struct PkShared {
   Fx part[3][NT / 32];
   double out[6];
   int ok;
-  ulonglong2 slots[2][MODE == kPkCluster ? kPkCluster16 : 1][4];  // cluster: slots written by the peers
+  ulonglong2 slots[2][MODE == kPkCluster ? kPkCluster16 : 1][kPkWords + 1];  // cluster: slots written by the peers
 };
 
 template <int NT>
@@ -183,6 +187,7 @@ __device__ __forceinline__ bool pk_step(const double* v, PkShared<NT, MODE>& sh,
     return true;
   }
   constexpr int NF = NV > 0 ? NV : 1;  // NV = 0: a barrier only
+  static_assert(NF <= kPkWords, "a slot holds the values of one step");
   Fx f[NF] = {};
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
@@ -207,10 +212,10 @@ __device__ __forceinline__ bool pk_step(const double* v, PkShared<NT, MODE>& sh,
       if (lane < G) {
         const uint32_t r = pk_mapa(a, lane);
 #pragma unroll
-        for (int k = 0; k < NF; ++k) pk_put_peer(r + 16 * k, pk_word(f[k], seq));
+        for (int k = 0; k < kPkWords; ++k) pk_put_peer(r + 16 * k, pk_word(k < NF ? f[k < NF ? k : 0] : Fx{0, 1}, seq));
       }
-    } else if (lane < NF) {
-      Fx mine = f[0];
+    } else if (lane < kPkWords) {
+      Fx mine = lane == 0 ? f[0] : Fx{0, 1};
       if (NF > 1 && lane == 1) mine = f[NF > 1 ? 1 : 0];
       if (NF > 2 && lane == 2) mine = f[NF > 2 ? 2 : 0];
       pk_put(base + me * kPkSlot + lane, pk_word(mine, seq));
@@ -486,7 +491,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
   rows.init(a, sm + (a.bj ? NT * RPT * sizeof(T) : 0));
   if constexpr (MODE == kPkCluster) {
     // no tag set; every block's slots are clear before a peer writes them
-    for (int i = threadIdx.x; i < 2 * kPkCluster16 * 4; i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
+    for (int i = threadIdx.x; i < 2 * kPkCluster16 * (kPkWords + 1); i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
     pk_cluster_barrier();
   }
   unsigned seq = 0;
@@ -743,7 +748,7 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
   rows.init(a, sm + (a.bj ? NT * RPT * sizeof(T) : 0));
   if constexpr (MODE == kPkCluster) {
     // no tag set; every block's slots are clear before a peer writes them
-    for (int i = threadIdx.x; i < 2 * kPkCluster16 * 4; i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
+    for (int i = threadIdx.x; i < 2 * kPkCluster16 * (kPkWords + 1); i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
     pk_cluster_barrier();
   }
   unsigned seq = 0;

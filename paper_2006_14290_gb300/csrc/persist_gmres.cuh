@@ -42,10 +42,12 @@ struct PkGmresShared {
 };
 
 // Totals over the grid of `count` <= 32 values, whose warp sums are in
-// sh.part, into sh.h.  False when a wait timed out (block-uniform).
+// sh.part, into sh.h.  False when a wait timed out (block-uniform).  `all`
+// (every cycle's first gather) also stores the words that it does not use, so
+// that no word keeps a tag from before its cycle, at most 4 x 31 steps ago.
 template <int NT, typename S>
-__device__ __forceinline__ bool pk_gather_sums(int count, S& sh, ulonglong2* sums, ulonglong2* totals, int* err,
-                                               unsigned& seq) {
+__device__ __forceinline__ bool pk_gather_sums(int count, bool all, S& sh, ulonglong2* sums, ulonglong2* totals,
+                                               int* err, unsigned& seq) {
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, G = gridDim.x, me = blockIdx.x;
@@ -57,6 +59,10 @@ __device__ __forceinline__ bool pk_gather_sums(int count, S& sh, ulonglong2* sum
   for (int i = w; i < count; i += NW) {
     const Fx f = NW > 1 ? warp_fx_sum(lane < NW ? sh.part[i][lane] : Fx{0, 1}) : sh.part[i][0];
     if (lane == 0) pk_put(sb + (size_t)i * kPkMaxBlocks + me, pk_word(f, seq));
+  }
+  if (all && w == 0 && lane >= count) {
+    pk_put(sb + (size_t)lane * kPkMaxBlocks + me, pk_word(Fx{0, 1}, seq));
+    if (lane % G == me) pk_put(tb + 2 * lane, pk_word(Fx{0, 1}, seq));
   }
   bool dead = false;
   // poll(i): until all the words that this lane reads carry the tag
@@ -202,7 +208,7 @@ __global__ void __launch_bounds__(NT) pk_gmres_kernel(PkGmresArgs<T, VT> ga) {
           const Fx f = warp_fx_sum(fx_of(s));
           if (lane == 0) gs.part[i][w] = f;
         }
-        if (!pk_gather_sums<NT>(j + 2 - pass, gs, ga.sums, ga.totals, a.err, seq)) {
+        if (!pk_gather_sums<NT>(j + 2 - pass, j == 0 && pass == 0, gs, ga.sums, ga.totals, a.err, seq)) {
           status = -1;
           break;
         }

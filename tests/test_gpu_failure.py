@@ -38,3 +38,25 @@ def test_bounded_wait_rejects_bad_limits(gko):
         with pytest.raises(G.GkoError) as e:
             G.gko_diag_bounded_wait(bad)
         assert e.value.status == G.INVALID_ARG
+
+
+@pytest.mark.parametrize("cluster,blocks", [(1, 2), (1, 7), (1, 16), (0, 2), (0, 33), (0, 152)])
+@pytest.mark.parametrize("values", [0, 1, 2, 3])
+def test_exchange_totals_and_slot_words(gko, cluster, blocks, values):
+    """The single-launch solvers' exchanges: every total and every published
+    entry is right over more steps than the 16-bit tags count, and no word of
+    a slot keeps the tag of an older step."""
+    G = gko
+    steps = 66_000 if blocks in (7, 33) else 500
+    out, cycles = G.gko_diag_exchange(bool(cluster), blocks, values, steps)
+    assert np.all(out[:, 0] == steps) and np.all(out[:, 1:] == 0), out
+    assert cycles > 0
+    G.gko_device_status()
+
+
+def test_exchange_check_rejects_bad_sizes(gko):
+    G = gko
+    for bad in ((True, 1, 1, 5), (True, 17, 1, 5), (False, 161, 1, 5), (True, 4, 4, 5), (True, 4, 1, 0)):
+        with pytest.raises(G.GkoError) as e:
+            G.gko_diag_exchange(*bad)
+        assert e.value.status == G.INVALID_ARG
