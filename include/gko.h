@@ -604,12 +604,17 @@ GKO_API int gko_diag_bounded_wait(int64_t cycles, int32_t *timed_out, void *stre
  * grid of 2 blocks up to one per SM, passes `steps` (1..1,000,000) steps that
  * each add `values` (1..3) numbers per thread over all blocks, or (0) publish
  * a vector, read a neighbour's part of it and pass a second barrier.
- * out[3 b .. 3 b + 2] (host): block b's steps, its wrong totals and vector
- * entries, and its slot words that do not carry the tag of their slot's last
- * step; the latter two must be 0.  *cycles_per_step: SM clock cycles of block
- * 0.  Synchronises `stream`; GKO_INVALID_ARG on sizes out of range. */
-GKO_API int gko_diag_exchange(int32_t cluster, int32_t blocks, int32_t values, int32_t steps, int32_t *out,
-                              double *cycles_per_step, void *stream);
+ * out[4 b .. 4 b + 3] (host): block b's steps, its wrong totals and vector
+ * entries, its slot words that do not carry the tag of their slot's last step
+ * (both must be 0), and whether it gave up.  *cycles_per_step: SM clock cycles
+ * of block 0.  Failure check: with leave_block >= 0 that block leaves at step
+ * `leave_step` as one whose wait ran out does; the others' waits for it run
+ * out after wait_cycles (0: the solvers' limit of 2^31, at most that), they
+ * give up too, and GKO_TIMEOUT stands in the device error word.  Synchronises
+ * `stream`; GKO_INVALID_ARG on arguments out of range. */
+GKO_API int gko_diag_exchange(int32_t cluster, int32_t blocks, int32_t values, int32_t steps, int32_t leave_block,
+                              int32_t leave_step, int64_t wait_cycles, int32_t *out, double *cycles_per_step,
+                              void *stream);
 
 #ifdef __cplusplus
 }

@@ -39,7 +39,7 @@ struct Ctl {
   // BiCGSTAB's half step
   double maxrr, delta;
   int half;
-  int pad2;
+  int gave_up;  // single-launch solves: a wait of some block timed out
 };
 
 __device__ __forceinline__ double wd(double v) { return v; }

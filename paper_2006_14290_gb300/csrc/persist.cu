@@ -69,7 +69,7 @@ template <typename T>
 int finish(const Ctl* c, cudaStream_t s, SolveOut* out) {
   Ctl* hc = host_ctl();
   GKO_TRY(read_ctl(c, hc, s));
-  if (hc->half) return fail(GKO_TIMEOUT, "single-launch solve: a grid reduction's wait timed out");
+  if (hc->gave_up) return fail(GKO_TIMEOUT, "single-launch solve: a grid reduction's wait timed out");
   out->status = hc->status;
   out->iterations = hc->iter;
   out->cycles = hc->cycles;
@@ -130,7 +130,8 @@ int launch(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const Solv
   a.c = cv.take<Ctl>(1);
   if (!cluster) a.slots = cv.take<ulonglong2>(2 * kPkMaxBlocks * kPkSlot);
   for (int k = 0; k < nvec; ++k) a.vec[k] = cv.take<T>((size_t)n);
-  if (!cluster) GKO_TRY_CUDA(cudaMemsetAsync(a.slots, 0, slot_bytes, s));
+  if (!cluster)  // the state and the slots behind it
+    GKO_TRY_CUDA(cudaMemsetAsync(a.c, 0, (size_t)((char*)a.slots - (char*)a.c) + slot_bytes, s));
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // the blocks cannot all be resident
     cudaGetLastError();
@@ -207,7 +208,7 @@ int run_gmres(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const S
       g.V = cv.take<T>((size_t)ld * (sp.restart + 1));
       g.ld = ld;
       g.m = sp.restart;
-      GKO_TRY_CUDA(cudaMemsetAsync(g.a.slots, 0, sizeof(ulonglong2) * words, s));
+      GKO_TRY_CUDA(cudaMemsetAsync(g.a.c, 0, (size_t)((char*)g.a.slots - (char*)g.a.c) + sizeof(ulonglong2) * words, s));
       void* args[] = {&g};
       const cudaError_t e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)G), dim3((unsigned)h.nt), args,
                                                         smem, s);

@@ -32,7 +32,9 @@
 //    for one to three more gathers and FMAs per matrix entry.
 //
 // Every wait is bounded (~1 s); a block that gives up records GKO_TIMEOUT and
-// leaves, and so do the others.
+// leaves (pk_leave), and so do the others, whose next wait for it runs out; in
+// a cluster every block stays until all have left, because its shared memory
+// may be read until then.
 #pragma once
 
 #include <algorithm>
@@ -144,6 +146,7 @@ struct PkShared {
   Fx part[3][NT / 32];
   double out[6];
   int ok;
+  unsigned left[MODE == kPkCluster ? kPkCluster16 : 1];  // cluster: the peers that are about to leave
   ulonglong2 slots[2][MODE == kPkCluster ? kPkCluster16 : 1][kPkWords + 1];  // cluster: slots written by the peers
 };
 
@@ -167,6 +170,46 @@ struct PkNothing {
   __device__ void operator()() const {}
 };
 
+// Kernel start.  Cluster: no tag and no flag set, and every block's words are
+// clear before a peer writes them.  *gave_up is the host's to clear in a grid.
+template <int NT, int MODE>
+__device__ __forceinline__ void pk_open(PkShared<NT, MODE>& sh, int* gave_up) {
+  if constexpr (MODE == kPkCluster) {
+    for (int i = threadIdx.x; i < 2 * kPkCluster16 * (kPkWords + 1); i += NT)
+      (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
+    if (threadIdx.x < kPkCluster16) sh.left[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *gave_up = 0;
+    pk_cluster_barrier();
+  }
+}
+
+// Kernel end, after a block's last access to another block's shared memory;
+// dead: one of its waits ran out.  Cluster: the block tells every peer and
+// passes cluster barriers until all have told it.  When all end together that
+// is one barrier.  A block that gives up is ahead of the others, who may still
+// pass barriers of their own and read its vectors: they find it here, its
+// shared memory alive, until a wait for it has run out for each of them too.
+// All flags are set before their writers' next arrival, so nobody reads or
+// writes a peer once one block has left.
+template <int NT, int MODE>
+__device__ __forceinline__ void pk_leave(PkShared<NT, MODE>& sh, bool dead, int* gave_up) {
+  if (dead && threadIdx.x == 0) *gave_up = 1;
+  if constexpr (MODE == kPkCluster) {
+    const unsigned G = gridDim.x;
+    if (threadIdx.x < G)
+      asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(
+                       pk_mapa(pk_smem(&sh.left[blockIdx.x]), threadIdx.x)),
+                   "r"(1u)
+                   : "memory");
+    unsigned told = 1u;
+    do {
+      pk_cluster_barrier();
+      if (threadIdx.x < G)
+        asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(told) : "r"(pk_smem(&sh.left[threadIdx.x])) : "memory");
+    } while (!__syncthreads_and(told != 0u));
+  }
+}
+
 // Sum of NV <= 3 values per thread over all blocks (NV = 0: a barrier); thread 0 of every block then
 // runs fin(totals, out) and the block reads out[] from sh.out.  `pre` runs in
 // thread 0 while the values travel.  False when a wait timed out
@@ -179,11 +222,10 @@ struct PkNothing {
 // read before the next step's first block barrier.
 template <int NT, int MODE, int PUB, int NV, typename F, typename P = PkNothing>
 __device__ __forceinline__ bool pk_step(const double* v, PkShared<NT, MODE>& sh, ulonglong2* slots, int* err,
-                                        unsigned& seq, F fin, P pre = P{}) {
+                                        unsigned& seq, F fin, P pre = P{}, long long wait = kPkWait) {
   constexpr unsigned kAll = 0xffffffffu;
   if constexpr (MODE == kPkCluster && NV == 0 && PUB != kPubGlobal) {
-    // the hardware barrier; a peer that gave up has left and is not waited for
-    pk_cluster_barrier();
+    pk_cluster_barrier();  // the hardware barrier; a peer that gave up passes it in pk_leave
     return true;
   }
   constexpr int NF = NV > 0 ? NV : 1;  // NV = 0: a barrier only
@@ -241,7 +283,7 @@ __device__ __forceinline__ bool pk_step(const double* v, PkShared<NT, MODE>& sh,
         for (int k = 0; k < NF; ++k) ready = ready && pk_tagged(w[i][k], seq);
       if (__all_sync(kAll, ready)) break;
       if (spins == 64) t0 = clock64();
-      if (spins > 64 && clock64() - t0 > kPkWait) dead = true;
+      if (spins > 64 && clock64() - t0 > wait) dead = true;
       if (__any_sync(kAll, dead)) {
         dead = true;
         break;
@@ -489,11 +531,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
   unsigned char* sm = smem_raw + (MODE == kPkCluster ? kPkClusterVecs * NT * RPT * sizeof(T) : 0);
   const PkPrecond<T, VT, NT, RPT> pre{reinterpret_cast<T*>(sm)};
   rows.init(a, sm + (a.bj ? NT * RPT * sizeof(T) : 0));
-  if constexpr (MODE == kPkCluster) {
-    // no tag set; every block's slots are clear before a peer writes them
-    for (int i = threadIdx.x; i < 2 * kPkCluster16 * (kPkWords + 1); i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
-    pk_cluster_barrier();
-  }
+  pk_open(sh, &a.c->gave_up);
   unsigned seq = 0;
   const bool pc = a.d != nullptr || a.bj != nullptr;
   // vector 0: FLY z = M^-1 r, else p; FLY: vectors 1 and 2 p, alternating
@@ -718,11 +756,10 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
     a.c->status = status < 0 ? kNotConverged : status;
     a.c->iter = it;
     a.c->cycles = 0;
-    a.c->half = status < 0 ? 1 : 0;  // 1: a wait timed out
     a.c->nb = nb;
     a.c->rr = rr_true;
   }
-  if constexpr (MODE == kPkCluster) pk_cluster_barrier();  // no block's shared memory goes while it may be read
+  pk_leave(sh, status < 0, &a.c->gave_up);
 }
 
 // ----------------------------------------------------------- BiCGSTAB --
@@ -746,11 +783,7 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
   unsigned char* sm = smem_raw + (MODE == kPkCluster ? kPkClusterVecs * NT * RPT * sizeof(T) : 0);
   const PkPrecond<T, VT, NT, RPT> pre{reinterpret_cast<T*>(sm)};
   rows.init(a, sm + (a.bj ? NT * RPT * sizeof(T) : 0));
-  if constexpr (MODE == kPkCluster) {
-    // no tag set; every block's slots are clear before a peer writes them
-    for (int i = threadIdx.x; i < 2 * kPkCluster16 * (kPkWords + 1); i += NT) (&sh.slots[0][0][0])[i] = make_ulonglong2(0ull, 0ull);
-    pk_cluster_barrier();
-  }
+  pk_open(sh, &a.c->gave_up);
   unsigned seq = 0;
   const bool pc = a.d != nullptr;  // FLY gatherers apply it
   const bool reliable = REL && a.val64 != nullptr;
@@ -1137,11 +1170,10 @@ __global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
     a.c->status = status < 0 ? kNotConverged : status;
     a.c->iter = it;
     a.c->cycles = cycles;
-    a.c->half = status < 0 ? 1 : 0;  // 1: a wait timed out
     a.c->nb = nb;
     a.c->rr = rr_true;
   }
-  if constexpr (MODE == kPkCluster) pk_cluster_barrier();  // no block's shared memory goes while it may be read
+  pk_leave(sh, status < 0, &a.c->gave_up);
 }
 
 // -------------------------------------------------------------- launch --

@@ -354,10 +354,10 @@ __global__ void __launch_bounds__(NT) pk_gmres_kernel(PkGmresArgs<T, VT> ga) {
     a.c->status = status < 0 ? kNotConverged : status;
     a.c->iter = it;
     a.c->cycles = cycles;
-    a.c->half = status < 0 ? 1 : 0;  // 1: a wait timed out
     a.c->nb = nb;
     a.c->rr = rr_true;
   }
+  pk_leave(sh, status < 0, &a.c->gave_up);
 }
 
 template <typename T, typename VT>

@@ -85,7 +85,7 @@ SIGNATURES = {
     "gko_bench_fma": (C.c_int, [C.c_int, _I32, _P, C.c_int64, _P]),
     "gko_bench_gather": (C.c_int, [C.c_int, _I32, _P, _I32, _P, C.c_int64, _P]),
     "gko_diag_bounded_wait": (C.c_int, [C.c_int64, C.POINTER(C.c_int32), _P]),
-    "gko_diag_exchange": (C.c_int, [_I32, _I32, _I32, _I32, _P, C.POINTER(_D), _P]),
+    "gko_diag_exchange": (C.c_int, [_I32, _I32, _I32, _I32, _I32, _I32, _I64, _P, C.POINTER(_D), _P]),
     "gko_dot": (C.c_int, [_I64, _P, _P, C.POINTER(_D), _P]),
     "gko_nrm2": (C.c_int, [_I64, _P, C.POINTER(_D), _P]),
     "gko_axpy": (C.c_int, [_I64, _D, _P, _P, _P]),
@@ -398,12 +398,13 @@ def gko_diag_bounded_wait(cycles: int, stream=None) -> bool:
     return bool(t.value)
 
 
-def gko_diag_exchange(cluster: bool, blocks: int, values: int, steps: int, stream=None):
-    """(per block: steps, wrong values, stale words; cycles a step) of the
-    single-launch solvers' exchanges."""
-    out, cycles = np.zeros((max(blocks, 0), 3), np.int32), C.c_double()
-    _check(lib().gko_diag_exchange(int(cluster), blocks, values, steps, _hptr(out), C.byref(cycles), _stream(stream)),
-           "gko_diag_exchange")
+def gko_diag_exchange(cluster: bool, blocks: int, values: int, steps: int, leave_block=-1, leave_step=-1,
+                      wait_cycles=0, stream=None):
+    """(per block: steps, wrong values, stale words, gave up; cycles a step)
+    of the single-launch solvers' exchanges."""
+    out, cycles = np.zeros((max(blocks, 0), 4), np.int32), C.c_double()
+    _check(lib().gko_diag_exchange(int(cluster), blocks, values, steps, leave_block, leave_step, wait_cycles,
+                                   _hptr(out), C.byref(cycles), _stream(stream)), "gko_diag_exchange")
     return out, cycles.value
 
 

@@ -49,7 +49,7 @@ def test_exchange_totals_and_slot_words(gko, cluster, blocks, values):
     G = gko
     steps = 66_000 if blocks in (7, 33) else 500
     out, cycles = G.gko_diag_exchange(bool(cluster), blocks, values, steps)
-    assert np.all(out[:, 0] == steps) and np.all(out[:, 1:] == 0), out
+    assert np.all(out == [steps, 0, 0, 0]), out
     assert cycles > 0
     G.gko_device_status()
 
@@ -60,3 +60,25 @@ def test_exchange_check_rejects_bad_sizes(gko):
         with pytest.raises(G.GkoError) as e:
             G.gko_diag_exchange(*bad)
         assert e.value.status == G.INVALID_ARG
+
+
+@pytest.mark.parametrize("cluster,blocks", [(True, 2), (True, 7), (True, 16), (False, 2), (False, 33)])
+@pytest.mark.parametrize("values", [0, 1, 3])
+@pytest.mark.parametrize("leave_step", [0, 5, 49])
+def test_exchange_ends_when_a_block_leaves(gko, cluster, blocks, values, leave_step):
+    """A block leaves in the middle (its peers may be in a barrier, and in a
+    cluster may read its shared memory later): the others' waits run out, all
+    blocks end, the time-out is recorded and the context keeps working."""
+    G = gko
+    G.gko_device_status()
+    out, _ = G.gko_diag_exchange(cluster, blocks, values, 50, blocks // 2, leave_step, 2_000_000)  # 1 ms
+    assert out[blocks // 2, 0] == leave_step and np.all(out[:, 3] == 1), out
+    assert np.all(out[:, 0] >= leave_step) and np.all(out[:, 0] <= 50), out
+    if values:
+        assert np.all(out[:, 0] == leave_step), out
+    with pytest.raises(G.GkoError) as e:
+        G.gko_device_status()
+    assert e.value.status == G.TIMEOUT
+    out, _ = G.gko_diag_exchange(cluster, blocks, values, 50)
+    assert np.all(out == [50, 0, 0, 0]), out
+    G.gko_device_status()
