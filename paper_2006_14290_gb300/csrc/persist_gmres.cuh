@@ -10,7 +10,7 @@
 // value i is added by block i mod G alone and comes back as one word, since
 // every block polling G x (j + 2) slots would be quadratic.  The next basis
 // vector is published unscaled with the norm's exchange and A w is scaled
-// instead of w, so no exchange stands between the norm and the next SpMV.
+// instead of w (PkScaled), so no exchange stands between the norm and the next SpMV.
 // Each thread keeps its rows of the basis to itself in global memory (its own
 // loads and stores only); the Hessenberg column, rotations and back
 // substitution are the same few operations in warp 0 of every block.
@@ -114,6 +114,27 @@ __device__ __forceinline__ bool pk_gather_sums(int count, bool all, S& sh, ulong
   return sh.ok != 0;
 }
 
+// The product A (c w) of a published, unscaled w with a factor c.  FP64: (A w)
+// times c; w . w and (A v) . (A v) were representable, so A w is.  FP32 holds
+// norms down to 2^-126 but not their product with the entries of a small A
+// (||w|| = 2^-100, ||A|| = 2^-40), so there the gathered w is first brought to
+// about 1 by the power of two below c, exactly, and the rest of c follows: bit
+// for bit the same where neither form leaves the range.
+template <typename T>
+struct PkScaled {
+  int k;  // FP32: w is taken as 2^k w
+  Lin<T> back;
+  static __device__ __forceinline__ int power(double c) {
+    if (sizeof(T) == 8) return 0;
+    return min(max((int)(((unsigned)__double2hiint(c) >> 20) & 0x7ffu) - 1023, -126), 127);
+  }
+  static __device__ __forceinline__ double rest(double c, int k) {
+    return sizeof(T) == 8 ? c : c * __hiloint2double((1023 - k) << 20, 0);
+  }
+  __device__ __forceinline__ explicit PkScaled(double c) : k(power(c)), back(pk_lin<T>(pk_pack<T>(rest(c, k)))) {}
+  __device__ __forceinline__ T in(T w) const { return sizeof(T) == 8 ? w : w * __int_as_float((k + 127) << 23); }
+};
+
 template <typename T, typename VT, int NT, int RPT, bool ST>
 __global__ void __launch_bounds__(NT) pk_gmres_kernel(PkGmresArgs<T, VT> ga) {
   constexpr int MODE = kPkGrid, U = 8;
@@ -180,6 +201,7 @@ __global__ void __launch_bounds__(NT) pk_gmres_kernel(PkGmresArgs<T, VT> ga) {
     if (threadIdx.x <= kPkRestart) gs.g[threadIdx.x] = threadIdx.x == 0 ? sh.out[2] : 0.0;
     double inv = sh.out[1];
     Lin<T> sc = pk_lin<T>(pk_pack<T>(inv));
+    PkScaled<T> pr(inv);
     int k = 0;
     bool end = false, broke = false, estimate = false;
     known = false;
@@ -190,7 +212,7 @@ __global__ void __launch_bounds__(NT) pk_gmres_kernel(PkGmresArgs<T, VT> ga) {
       for (int u = 0; u < RPT; ++u) {
         const int32_t i = rows.row[u];
         if (i >= 0) ga.V[(int64_t)j * ga.ld + i] = sc.scale(wj[u]);
-        nw[u] = sc.scale((T)rows.template dot<U>(a, u, at(0), one));
+        nw[u] = pr.back.scale((T)rows.template dot<U>(a, u, at(0), [&](T v) { return pr.in(v); }));
       }
 #pragma unroll
       for (int u = 0; u < RPT; ++u) wj[u] = rows.row[u] >= 0 ? nw[u] : T(0);
@@ -262,7 +284,7 @@ __global__ void __launch_bounds__(NT) pk_gmres_kernel(PkGmresArgs<T, VT> ga) {
               gs.g[j + 1] = -sj * gj;
               gs.g[j] = cj * gj;
               if (hn == 0.0 || fabs(gs.g[j + 1]) <= tol) o[1] = 1.0;
-              o[2] = pk_pack<T>(1.0 / hn);
+              o[2] = 1.0 / hn;
             })) {
           status = -1;
           break;
@@ -275,7 +297,9 @@ __global__ void __launch_bounds__(NT) pk_gmres_kernel(PkGmresArgs<T, VT> ga) {
       broke = sh.out[1] == 2.0;
       estimate = sh.out[1] == 1.0;
       k = broke ? j : j + 1;
-      sc = pk_lin<T>(sh.out[2]);
+      inv = sh.out[2];
+      sc = pk_lin<T>(pk_pack<T>(inv));
+      pr = PkScaled<T>(inv);
       end = broke || estimate || it >= a.maxit || j + 1 == ga.m;
     }
     if (status != kRun) break;

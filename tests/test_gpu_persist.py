@@ -252,3 +252,22 @@ def test_iteration_cap_near_attainable_accuracy(gko, name, n, fmt, precond):
         assert res.iterations <= cap and res.status in (G.NOT_CONVERGED, G.BREAKDOWN), (cap, res)
         true = np.linalg.norm(b - O.spmv_csr(A, x)) / np.linalg.norm(b)
         assert abs(true - res.rel_residual) <= 1e-13
+
+
+@pytest.mark.parametrize("ka,kb", [(0, 0), (-45, -75), (45, 60), (-45, 60)])
+@pytest.mark.parametrize("n", [700, 9001])
+def test_gmres_mixed_at_any_scale_of_matrix_and_right_hand_side(gko, n, ka, kb):
+    """Mixed GMRES on 2^ka A x = 2^kb b: residuals and entries are FP32
+    numbers, their products need not be; the same iterations and digits as
+    without the powers of two."""
+    G = gko
+    A = banded_system(n, 7, False, n)
+    b = np.random.default_rng(1).uniform(-1, 1, n)
+    As = I.Csr(A.n_rows, A.n_cols, A.row_ptr, A.col, np.ldexp(A.val, ka), A.name)
+    runs = []
+    for M, rhs in ((G.from_csr(A), b), (G.from_csr(As), np.ldexp(b, kb))):
+        xd = dev(np.zeros(n))
+        res = G.gko_solve_gmres(M, dev(rhs), xd, 1e-12, 3000, G.opts(precision=G.PRECISION_MIXED_F32))
+        assert res.status == G.OK, res
+        runs.append((res.iterations, host(xd)))
+    assert runs[1][0] == runs[0][0] and np.array_equal(runs[1][1], np.ldexp(runs[0][1], kb - ka))
