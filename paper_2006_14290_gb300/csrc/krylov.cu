@@ -106,9 +106,9 @@ __device__ __forceinline__ void vec_loop(int64_t n, bool aligned, VF vf, SF sf) 
   for (int64_t i = done + tid; i < n; i += nth) sf(i);
 }
 
-template <int NV, typename Op>
+template <int NV, bool TREE = false, typename Op>
 __device__ __forceinline__ void reduce_op(double (&v)[NV], RedWs ws, Op op) {
-  grid_reduce<256, NV>(v, ws.partials, ws.counter, blockIdx.x, gridDim.x, op);
+  grid_reduce<256, NV, TREE>(v, ws.partials, ws.counter, blockIdx.x, gridDim.x, op);
 }
 
 #define GKO_GRID_LOOP(i, n) \
@@ -415,7 +415,7 @@ struct CgUpdateOp {
 // alpha = rho / (p.q); x += alpha p; r -= alpha q; reduces r.r and, with
 // the Jacobi inverse diagonal d (PC), r.z for z = d r.  BJ: r.r only, the
 // step scalars left to the block-Jacobi kernel that follows.
-template <typename T, bool PC, bool BJ = false>
+template <typename T, bool PC, bool BJ = false, bool TREE = false>
 __global__ void __launch_bounds__(256, 4) cg_update_kernel(int64_t n, T* __restrict__ x, T* __restrict__ r,
                                                         const T* __restrict__ p, const T* __restrict__ q, Ctl* c,
                                                         RedWs ws, const T* __restrict__ d) {
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(256, 4) cg_update_kernel(int64_t n, T* __restr
           if (PC) acc[NV - 1] = __fma_rn(rw, wd(d[i] * ri), acc[NV - 1]);
         });
   }
-  reduce_op<NV>(acc, ws, CgUpdateOp<NV, BJ>{c});
+  reduce_op<NV, TREE>(acc, ws, CgUpdateOp<NV, BJ>{c});
 }
 
 // p = z + beta p, z = d r with the Jacobi inverse diagonal (PC), else r
@@ -1255,6 +1255,14 @@ struct BatchGraph {
 };
 constexpr int kGraphIters = 16;  // iterations per replayed batch
 
+// Rows from which unpreconditioned FP64 CG sums r.r as an FP64 tree
+// (block_tree_n).  us an iteration, tree and integer sums, 7-point: 88^3 48.6
+// and 47.2, 96^3 55.3 and 55.6, 112^3 74.1 and 78.2, 128^3 95.7 and 99.5, 144^3
+// 130.5 and 137.1, 160^3 162.2 and 164.1, 256^3 the same.  With a preconditioner,
+// in FP32 and in BiCGSTAB the integer sums are the faster or the same (Jacobi,
+// 128^3: 110.0 and 107.3; BiCGSTAB within 2% either way).
+constexpr int64_t kTreeRows = 1 << 20;
+
 // One Krylov solve on the device.  A: matrix whose value type matches T
 // (double: F64; float: F32/BF16).  b: FP64 right-hand side; x: T vector,
 // x0 on entry (x_zero: treat x0 as zero without reading it).
@@ -1350,6 +1358,7 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
     // programmatic serialization (PdlScope), so its dispatch overlaps the
     // drain of the one before; each waits for that one before touching memory.
     const dim3 B256(256);
+    const bool tree = sizeof(T) == 8 && n >= kTreeRows;
     auto enqueue = [&](int count) -> int {
       PdlScope pdl(true);
       for (int it = 0; it < count; ++it) {
@@ -1366,8 +1375,8 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
             GKO_TRY_CUDA(launch_k(cg_update_kernel<T, true>, dim3(rg), B256, 0, s, n, x, r, p, q, c, ws, dinv));
             GKO_TRY_CUDA(launch_k(cg_p_kernel<T, true>, dim3(vg), B256, 0, s, n, r, p, c, dinv));
           } else {
-            GKO_TRY_CUDA(launch_k(cg_update_kernel<T, false>, dim3(rg), B256, 0, s, n, x, r, p, q, c, ws,
-                                  (const T*)nullptr));
+            GKO_TRY_CUDA(launch_k(tree ? cg_update_kernel<T, false, false, sizeof(T) == 8> : cg_update_kernel<T, false>,
+                                  dim3(rg), B256, 0, s, n, x, r, p, q, c, ws, (const T*)nullptr));
             GKO_TRY_CUDA(launch_k(cg_p_kernel<T, false>, dim3(vg), B256, 0, s, n, r, p, c, (const T*)nullptr));
           }
         } else if (bj) {

@@ -379,3 +379,22 @@ def test_solver_workloads_full_size(gko, case):
         tr = true_rel_res(A, x, b)
         assert tr <= 1.01e-8 and abs(res.rel_residual - tr) <= 1e-11
         assert np.linalg.norm(x - 1.0) <= 1e-4 * np.sqrt(A.n_rows)
+
+
+@pytest.mark.parametrize("n", [(1 << 20) - 1, 1 << 20, (1 << 20) + 1])
+def test_cg_where_the_sums_change_form(gko, n):
+    """Unpreconditioned FP64 CG around 2^20 rows, where its block sums change
+    from integers to an FP64 tree: the oracle's iterate after 12 steps."""
+    G = gko
+    i = np.arange(n)
+    A = I.Csr(n, n, np.arange(0, 3 * n + 1, 3, dtype=np.int32)[: n + 1],
+              np.sort(np.stack([i, (i + 1) % n, (i - 1) % n], 1), 1).astype(np.int32).ravel(), None, "ring")
+    A.val = np.where(A.col == np.repeat(i, 3), 2.5, -1.0)
+    b = np.random.default_rng(0).uniform(-1, 1, n)
+    xd = dev(np.zeros(n))
+    res = G.gko_solve_cg(G.from_csr(A), dev(b), xd, 0.0, 12)
+    xo, ro = O.cg(A, b, tol=0.0, maxit=12)
+    assert res.iterations == ro.iterations == 12
+    assert np.linalg.norm(host(xd) - xo) <= 1e-12 * np.linalg.norm(xo)
+    true = np.linalg.norm(b - O.spmv_csr(A, xo)) / np.linalg.norm(b)
+    assert abs(res.rel_residual - true) <= 1e-12
