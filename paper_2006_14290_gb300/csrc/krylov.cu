@@ -954,6 +954,40 @@ __global__ void __launch_bounds__(256, 4) gm_multidot_kernel(int64_t n, int k, c
   }
 }
 
+// The same for small steps, one vector to a block and the chunks added by a
+// second launch, whose dispatch programmatic serialization hides: groups and
+// tickets cost more than they save where a block has little to add.  Grouped
+// and this, us per Arnoldi step (FP64, 7-point COO): 20^3, restart 30, 62.8 and
+// 53.8; 31^3, 30, 67.9 and 60.7; 45^3, 60, 105.7 and 98.1; 60^3, 30, 103.2 and
+// 97.6; from n * k = kSmallDot on the groups.  In FP32 they are the faster at
+// every size (20^3, restart 60: 60.8, with one vector to a block 69.8).
+constexpr int64_t kSmallDot = 3 << 20;
+constexpr int kSmallDotRows = 2048;
+constexpr int kSmallDotSlots = (int)(kSmallDot / kSmallDotRows) + kMaxRestart;
+
+template <typename T>
+__global__ void __launch_bounds__(256, 4) gm_dot_kernel(int64_t n, const T* __restrict__ V, int64_t ldv,
+                                                     const T* __restrict__ w, double* __restrict__ partials, Ctl* c,
+                                                     int pass) {
+  pdl_begin();
+  if (gated(&c->phase) || (pass == 1 && *(volatile int*)&c->noreorth)) return;
+  const T* v = V + (int64_t)blockIdx.y * ldv;
+  double acc = 0.0;
+  GKO_GRID_LOOP(i, n) acc = __fma_rn(wd(v[i]), wd(w[i]), acc);
+  const double t = block_sum<256>(acc);
+  if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = t;
+}
+
+__global__ void __launch_bounds__(256, 4) gm_dot_finish_kernel(int chunks, const double* __restrict__ partials,
+                                                            double* __restrict__ h, Ctl* c, int pass) {
+  pdl_begin();
+  if (gated(&c->phase) || (pass == 1 && *(volatile int*)&c->noreorth)) return;
+  double acc[1] = {0.0};
+  for (int i = threadIdx.x; i < chunks; i += 256) acc[0] += partials[blockIdx.x * chunks + i];
+  block_tree_n<256, 1>(acc);
+  if (threadIdx.x == 0) h[blockIdx.x] = acc[0];
+}
+
 struct StoreRr {
   Ctl* c;
   int decide;  // first pass: skip the second pass unless ||w|| fell below ||w0|| / sqrt(2)
@@ -1281,9 +1315,10 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
   const int bs = sp.bs;
   const size_t spmv_sb = spmv_scratch_bytes(A);
   const int slots = std::max(kMaxRestart, 4 * sm_count());  // partial sums of a multi-dot's group member
+  const size_t dot_slots = std::max<size_t>((size_t)kDotGroup * slots, kSmallDotSlots);
   const size_t bytes = 256 * 16 + sizeof(Ctl) + sizeof(double) * 3 * kDotSlots + 512 +
                        (size_t)nvec * (sizeof(T) * ((size_t)n + 64) + 320) + spmv_sb + 320 +
-                       sizeof(double) * ((size_t)(m + 1) * m + 6 * (m + 2) + (size_t)kDotGroup * slots) + 4096;
+                       sizeof(double) * ((size_t)(m + 1) * m + 6 * (m + 2) + dot_slots) + 4096;
   Scratch mem;
   GKO_TRY(mem.get(bytes, s));
   Carve cv{static_cast<char*>(mem.data())};
@@ -1482,7 +1517,7 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
     double* h1 = cv.take<double>(m + 2);
     double* h2 = cv.take<double>(m + 2);
     double* ny = cv.take<double>(m + 2);
-    double* mpart = cv.take<double>((size_t)kDotGroup * slots);
+    double* mpart = cv.take<double>(dot_slots);
     unsigned* dcount = cv.take<unsigned>(kMaxDotGroups);
     GKO_TRY_CUDA(cudaMemsetAsync(dcount, 0, sizeof(unsigned) * kMaxDotGroups, s));
     // ||b|| and the zero-b case through the common init kernel
@@ -1526,10 +1561,18 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
         // shrank ||w|| below ||w0|| / sqrt(2) (selective reorthogonalisation)
         for (int pass = 0; pass < 2; ++pass) {
           double* hp = pass == 0 ? h1 : h2;
-          // one wave of blocks, 1,024 rows of four vectors or more to a block
-          const int64_t blocks = std::max<int64_t>(j + 1, std::min<int64_t>((n + 4095) / 4096 * (j + 1), slots));
-          GKO_TRY_CUDA(launch_k(gm_multidot_kernel<T>, dim3((unsigned)blocks), dim3(256), 0, s, n,
-                                j + 1, (const T*)V, ld, (const T*)w, hp, mpart, dcount, c, pass));
+          if (sizeof(T) == 8 && n * (j + 1) <= kSmallDot) {
+            const int chunks = (int)((n + kSmallDotRows - 1) / kSmallDotRows);
+            GKO_TRY_CUDA(launch_k(gm_dot_kernel<T>, dim3((unsigned)chunks, (unsigned)(j + 1)), dim3(256), 0, s, n,
+                                  (const T*)V, ld, (const T*)w, mpart, c, pass));
+            GKO_TRY_CUDA(launch_k(gm_dot_finish_kernel, dim3(j + 1), dim3(256), 0, s, chunks, (const double*)mpart, hp,
+                                  c, pass));
+          } else {
+            // one wave of blocks, 1,024 rows of four vectors or more to a block
+            const int64_t blocks = std::max<int64_t>(j + 1, std::min<int64_t>((n + 4095) / 4096 * (j + 1), slots));
+            GKO_TRY_CUDA(launch_k(gm_multidot_kernel<T>, dim3((unsigned)blocks), dim3(256), 0, s, n,
+                                  j + 1, (const T*)V, ld, (const T*)w, hp, mpart, dcount, c, pass));
+          }
           GKO_TRY_CUDA(launch_k(gm_axpy_kernel<T, true>, dim3(rg), dim3(256), 0, s, n, j + 1, (const double*)hp,
                                 (const T*)V, ld, w, c, ws, pass));
         }
