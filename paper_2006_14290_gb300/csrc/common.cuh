@@ -124,6 +124,7 @@ struct CsrPlan {
   int64_t tile_start_at = 0;  // ... at this int32 offset
   int64_t tiles = 0;    // 0: the kernels with carries
   int32_t tile_width = 0;  // W
+  int32_t tile_len = 0;    // COO: longest row
   // COO handles: kind 1 runs the row-block kernel over the COO arrays, any
   // other kind the tiled segmented reduction.
   Buf coo_rb;          // int32[n_rb+1]     first COO entry of each row block of (128/S)*R rows

@@ -334,8 +334,8 @@ __global__ void tile_starts_kernel(int64_t n, int64_t tiles, int64_t width, cons
 }
 
 // Row-aligned tiles of a matrix (0: the kernels with carries, see spmv.cuh).
-static int64_t tile_count(int64_t n, int64_t nnz, int32_t max_len) {
-  if (nnz == 0 || max_len > kTileRowMax || (nnz > kTileNnzMax && nnz < kTileRowMean * n)) return 0;
+static int64_t tile_count(int64_t nnz, int32_t max_len, gko_dtype dtype) {
+  if (!tiles_worth(nnz, max_len, dtype)) return 0;
   const int64_t w = tile_width_for(max_len);
   return (nnz + w - 1) / w;
 }
@@ -344,7 +344,8 @@ static int64_t tile_count(int64_t n, int64_t nnz, int32_t max_len) {
 // its row indices (coo_row holds `nnz` of them, then tiles + 1 starts).
 static int build_tile_starts(gko_matrix m, const int32_t* rp, int64_t nnz, int32_t max_len, cudaStream_t s) {
   CsrPlan& p = m->plan;
-  p.tiles = tile_count(m->n_rows, nnz, max_len);
+  p.tiles = tile_count(nnz, max_len, GKO_F32);  // what FP32 wants includes what FP64 does
+  p.tile_len = max_len;
   if (!p.tiles) return GKO_OK;
   p.tile_start = m->coo_row;
   p.tile_width = tile_width_for(max_len);
@@ -356,8 +357,8 @@ static int build_tile_starts(gko_matrix m, const int32_t* rp, int64_t nnz, int32
 }
 
 // int32 words of a COO part's row indices and the tile starts behind them
-static int64_t coo_row_words(int64_t n, int64_t nnz, int32_t max_len) {
-  const int64_t t = tile_count(n, nnz, max_len);
+static int64_t coo_row_words(int64_t nnz, int32_t max_len) {
+  const int64_t t = tile_count(nnz, max_len, GKO_F32);
   return t ? (nnz + 3) / 4 * 4 + t + 1 : nnz;
 }
 
@@ -367,7 +368,7 @@ static int build_seg_rows(gko_matrix m, cudaStream_t s) {
   p.seg_tiles = 0;
   p.tiles = 0;
   if (p.kind != 3 || m->nnz == 0) return GKO_OK;
-  p.tiles = tile_count(m->n_rows, m->nnz, p.max_len);
+  p.tiles = tile_count(m->nnz, p.max_len, m->dtype);
   p.tile_width = p.tiles ? tile_width_for(p.max_len) : kCooTile;
   const int64_t tiles = p.tiles ? p.tiles : (m->nnz + kCooTile - 1) / kCooTile;
   GKO_TRY(alloc(sizeof(int32_t) * (tiles + 1), &p.seg_row));
@@ -376,6 +377,20 @@ static int build_seg_rows(gko_matrix m, cudaStream_t s) {
   GKO_TRY_CUDA(cudaGetLastError());
   GKO_TRY_CUDA(cudaStreamSynchronize(s));
   p.seg_tiles = tiles;
+  return GKO_OK;
+}
+
+// The nonzero split of a handle on src's pattern: shared, unless the value
+// types want different tiles.
+static int share_seg_rows(gko_matrix m, const gko_matrix_s* src, cudaStream_t s) {
+  CsrPlan& p = m->plan;
+  if (m->fmt == GKO_CSR && p.kind == 3 &&
+      tiles_worth(m->nnz, p.max_len, m->dtype) != tiles_worth(m->nnz, p.max_len, src->dtype))
+    return build_seg_rows(m, s);
+  p.seg_row = src->plan.seg_row;
+  p.seg_tiles = src->plan.seg_tiles;
+  p.tiles = src->plan.tiles;
+  p.tile_width = src->plan.tile_width;
   return GKO_OK;
 }
 
@@ -684,10 +699,7 @@ int gko_matrix_set_plan(gko_matrix m, int32_t kernel, int32_t S, int32_t R, int3
       q.chunk_start = m->plan.chunk_start;
       q.merge_x = m->plan.merge_x;
       q.merge_tiles = m->plan.merge_tiles;
-      q.seg_row = m->plan.seg_row;
-      q.seg_tiles = m->plan.seg_tiles;
-      q.tiles = m->plan.tiles;
-      q.tile_width = m->plan.tile_width;
+      GKO_TRY(share_seg_rows(kv.second, m, (cudaStream_t)stream));
     }
   }
   return GKO_OK;
@@ -793,7 +805,7 @@ int gko_matrix_convert_to_coo(gko_matrix csr, void* stream, gko_matrix* out) {
   m->plan.S = csr->plan.S;
   m->plan.R = csr->plan.R;
   m->plan.cap = std::min<int32_t>(csr->plan.cap, kCooRbMaxCap);
-  GKO_TRY(alloc(sizeof(int32_t) * coo_row_words(csr->n_rows, nnz, csr->plan.max_len), &m->coo_row));
+  GKO_TRY(alloc(sizeof(int32_t) * coo_row_words(nnz, csr->plan.max_len), &m->coo_row));
   GKO_TRY(alloc(sizeof(int32_t) * nnz, &m->coo_col));
   GKO_TRY(alloc(vs * nnz, &m->coo_val));
   GKO_TRY(build_tile_starts(m.get(), ptr<int32_t>(csr->row_ptr), nnz, csr->plan.max_len, s));
@@ -851,7 +863,7 @@ int gko_matrix_convert_to_hybrid(gko_matrix csr, int32_t ell_width, void* stream
   const size_t vs = dtype_size(csr->dtype);
   m->coo_nnz = tail;
   const int32_t tail_len = std::max<int32_t>(0, csr->plan.max_len - K);  // longest row of the tail
-  GKO_TRY(alloc(sizeof(int32_t) * coo_row_words(n, tail, tail_len), &m->coo_row));
+  GKO_TRY(alloc(sizeof(int32_t) * coo_row_words(tail, tail_len), &m->coo_row));
   GKO_TRY(build_tile_starts(m.get(), ptr<int32_t>(tptr), tail, tail_len, s));
   GKO_TRY(alloc(sizeof(int32_t) * tail, &m->coo_col));
   GKO_TRY(alloc(vs * tail, &m->coo_val));
@@ -910,12 +922,10 @@ int gko_matrix_convert_values(gko_matrix src, gko_dtype to, void* stream, gko_ma
   m->plan.chunk_start = src->plan.chunk_start;
   m->plan.merge_x = src->plan.merge_x;
   m->plan.merge_tiles = src->plan.merge_tiles;
-  m->plan.seg_row = src->plan.seg_row;
-  m->plan.seg_tiles = src->plan.seg_tiles;
+  GKO_TRY(share_seg_rows(m.get(), src, s));
   m->plan.tile_start = src->plan.tile_start;
   m->plan.tile_start_at = src->plan.tile_start_at;
-  m->plan.tiles = src->plan.tiles;
-  m->plan.tile_width = src->plan.tile_width;
+  m->plan.tile_len = src->plan.tile_len;
   m->plan.coo_rb = src->plan.coo_rb;
   m->plan.coo_rb_n = src->plan.coo_rb_n;
   m->K = src->K;

@@ -19,10 +19,10 @@ size_t spmv_scratch_bytes(const gko_matrix_s* A) {
     case GKO_SELLP:
       return 0;
     case GKO_COO:
-      if (A->plan.kind == 1 || A->plan.tiles) return 0;
+      if (A->plan.kind == 1 || coo_tiles(A)) return 0;
       return at * 2 * (size_t)((A->coo_nnz + kCooTile - 1) / kCooTile);
     case GKO_HYBRID:
-      if (A->plan.tiles) return 0;
+      if (coo_tiles(A)) return 0;
       return at * 2 * (size_t)((A->coo_nnz + kCooTile - 1) / kCooTile);
   }
   return 0;

@@ -54,17 +54,33 @@ constexpr int kCooTile = kCooThreads * kCooItems;
 // block's window is the kCooTile entries from t W on; W leaves room for the
 // rest of the tile's last row where rows are short, so the window nearly
 // always holds the whole tile.
-// Used where the longest row is at most kTileRowMax (one block adds what a
-// row has behind the window: with rows of 10,000 the power-law matrices took
-// 62-103 us instead of 54-79) and where the launch and the workspace that go
-// away are worth more than the overlapping windows and the stores' bounds:
-// up to kTileNnzMax nonzeros (COO on 64^2 11.6 -> 8.8 us, CSR on 5,000
-// power-law rows 14.4 -> 10.2; 27-point COO on 128^3, 55.7 M, 189 -> 197), or
-// rows of kTileRowMean on average, few ends to bound (banded, 39.4 M: 144.6
-// -> 139.6).
+// Used where the launch and the workspace that go away (6-8 us) are worth more
+// than the overlapping windows and the rest of a row behind the window, which
+// one block adds.  Both grow with the nonzeros, the latter also with the
+// longest row L (at most kTileRowMax), in FP64 twice as fast as in FP32.
+// Speedup of COO over the kernels with carries, FP64 / FP32, rows of L entries
+// next to the diagonal:
+//   L = 27    4 M 1.28 / 1.27   8 M 1.16 / 1.19   16 M 1.05 / 1.02   40 M 1.04 / 0.91
+//   L = 96    4 M 1.20 / 1.31   6 M 1.15 / 1.16    8 M 1.13 / 1.15
+//   L = 200   1 M 1.24 / 1.32   2 M 1.09 / 1.31    4 M 1.00 / 1.22    8 M 0.93 / 1.15
+//   L = 500   1 M 1.18 / 1.24   2 M 1.10 / 1.18    4 M 0.92 / 1.23    8 M 0.85 / 1.10
+//   L = 1800  1 M 1.16 / 1.40   2 M 1.04 / 1.18    4 M 0.88 / 1.13    8 M 0.80 / 0.97
+// Random columns, rows of 1..L: FP64 L = 64 4 M 1.09, 8 M 0.95; L = 500 2 M 1.04,
+// 4 M 0.98; FP32 L = 300 8 M 1.05; L = 900 3 M 1.10, 8 M 1.06.  CSR gains 3-10%
+// less than COO.
 constexpr int32_t kTileRowMax = 2048;
-constexpr int64_t kTileNnzMax = 1 << 23;
-constexpr int64_t kTileRowMean = 32;
+inline bool tiles_worth(int64_t nnz, int32_t max_len, gko_dtype dtype) {
+  if (nnz == 0 || max_len > kTileRowMax) return false;
+  if (dtype == GKO_F64) {
+    if (max_len <= 48) return nnz <= 1 << 23;
+    return nnz <= 3 << 19 || (nnz <= 3 << 21 && nnz * max_len <= 9ll << 26);
+  }
+  return nnz <= 1 << 21 || (nnz <= 1 << 23 && nnz * max_len <= 3ll << 30);
+}
+// COO handles and hybrid tails carry the tile starts where any type wants them.
+inline bool coo_tiles(const gko_matrix_s* A) {
+  return A->plan.tiles > 0 && tiles_worth(A->coo_nnz, A->plan.tile_len, A->dtype);
+}
 inline int32_t tile_width_for(int32_t max_len) {
   const int32_t room = max_len < 64 ? max_len : 64;
   return (kCooTile - room) / 8 * 8;

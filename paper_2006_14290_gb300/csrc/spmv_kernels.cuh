@@ -1792,7 +1792,7 @@ struct SpmvImpl {
     AT* carry = static_cast<AT*>(scratch);
     CooArgs<VT, XT> a{A->n_rows, A->n_cols, nnz, ptr<int32_t>(A->coo_row), ptr<int32_t>(A->coo_col),
                       ptr<VT>(A->coo_val), x, y, alpha, beta, alpha == AT(1) && beta == AT(0)};
-    if (A->plan.tiles) {
+    if (coo_tiles(A)) {
       const cudaError_t e = accum ? coo_tile_launch<VT, XT, true>(a, A->plan, gate, s)
                                   : coo_tile_launch<VT, XT, false>(a, A->plan, gate, s);
       GKO_TRY_CUDA(e);

@@ -73,7 +73,7 @@ extern "C" int gko_spmv_coo_noalloc(const double* alpha, gko_matrix A, const dou
   }
   CooArgs<double, double> args{A->n_rows, A->n_cols, nnz, ptr<int32_t>(A->coo_row), ptr<int32_t>(A->coo_col),
                                ptr<double>(A->coo_val), x, y, a, b, a == 1.0 && b == 0.0};
-  if (A->plan.tiles) {  // row-aligned tiles: no carries
+  if (coo_tiles(A)) {  // row-aligned tiles: no carries
     const cudaError_t e = coo_tile_launch<double, double, false>(args, A->plan, nullptr, s);
     GKO_TRY_CUDA(e);
     return GKO_OK;

@@ -85,3 +85,33 @@ def test_deferred_row_sums(gko, S, extra, waves):
     yd = dev(np.zeros(n))
     d = G.gko_spmv_dot(M, dev(x), yd)  # x . (A x)
     assert abs(d - x @ yo) <= 1e-13 * (np.abs(x) @ np.abs(yo)) + np.abs(x) @ bound
+
+
+# both sides of the rule's lines: FP64 3 * 2^19 and 9 * 2^26 / L, FP32 2^21 and 3 * 2^30 / L, 2^23 for stencils
+@pytest.mark.parametrize("L,rows", [(2000, 786), (2000, 787), (200, 15099), (200, 15100), (48, 174762), (48, 174763),
+                                    (2000, 1048), (2000, 1049), (600, 8947), (600, 8948)])
+@pytest.mark.parametrize("fmt", ["coo", "split", "hybrid0"])
+def test_both_sides_of_the_tile_rule(gko, L, rows, fmt):
+    """FP64, and the FP32 handle made from it (which may tile where FP64
+    does not), before and after the plan is set again."""
+    G = gko
+    A = I.rows_csr([L] * rows, 3000, np.random.default_rng(L))
+    M = G.from_csr(A)
+    if fmt == "split":
+        M.set_plan(3, 1, 1, 1024)
+    else:
+        M = G.gko_matrix_convert_to_coo(M) if fmt == "coo" else G.gko_matrix_convert_to_hybrid(M, 0)
+    rng = np.random.default_rng(5)
+    x, y0 = rng.uniform(-1, 1, A.n_cols), rng.uniform(-1, 1, A.n_rows)
+    yd = dev(y0)
+    G.gko_spmv(-0.75, M, dev(x), 1.5, yd)
+    check_spmv_f64(host(yd), A, x, -0.75, 1.5, y0)
+    x32, v32 = x.astype(np.float32), A.val.astype(np.float32).astype(np.float64)
+    M32 = G.gko_matrix_convert_values(M, G.F32)
+    for again in range(2):
+        yd = dev(y0, np.float32)
+        G.gko_spmv(-0.75, M32, dev(x32), 1.5, yd)
+        check_spmv_f32(host(yd), A, x32.astype(np.float64), -0.75, 1.5, y0.astype(np.float32).astype(np.float64), v32)
+        if fmt != "split":
+            break
+        M32.set_plan(3, 1, 1, 1024)
