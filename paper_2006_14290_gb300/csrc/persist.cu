@@ -33,6 +33,40 @@ const Buf& vals_of(const gko_matrix_s* A) {
   return A->fmt == GKO_CSR ? A->val : A->fmt == GKO_ELL ? A->ell_val : A->sellp_val;
 }
 
+// Lines between these kernels and the multi-kernel solve, by the longest row K.
+// Figures: speedup over the multi-kernel solve, band matrix / random columns,
+// FP64, CSR unless ELL is said (whose multi-kernel product is the faster one).
+//
+// A published vector costs an exchange, recomputing it (kPkFly) one gather more
+// per entry in CG, two and one in BiCGSTAB's products.  CG, 14,000 rows, kPkFly /
+// published: K = 7 2.9 / 2.5, 17 2.7 / 2.6, 65 1.7 / 2.3; random columns, K = 65 1.4 / 1.9.
+// BiCGSTAB, 25,000 rows: K = 7 2.6 / 2.5, 17 2.2 / 2.7, 65 1.4 / 2.3; random 0.9 / 1.7.
+constexpr int64_t kPkFlyRow = 16;
+// In a cluster 16 SMs read each other's shared memory, fast from neighbours, not
+// at random: CG, 4,096 rows, cluster / published, K = 17 3.2 / 2.4, 27 3.0 / 2.2, 49 2.4 / 1.9;
+// random 1.5 / 2.3, 1.0 / 2.1, 0.6 / 1.8.  More entries than this take the grid; in
+// FP32 CG, whose grid shapes are as fast there, fewer (the second line).
+constexpr int64_t kPkClusterEntries = 7 << 14, kPkClusterEntriesCg32 = 1 << 16;
+// Entries that do not fit in shared memory are read from the matrix, a row to a
+// lane, which long rows and few SMs make slow:
+//   a row a thread:  CG 38,000 rows K = 129 2.0 / 1.5, 257 1.1 / 1.2   25,000 257 1.7 / 1.3
+//                    14,000 201 1.3 / 0.9, 401 1.2 / 0.9   9,700 401 0.6 / 0.6; ELL 1.6 / 1.1
+//   two rows:        CG 79,000 K = 97 1.3 / 1.1   120,000 97 1.3 / 1.4; ELL 79,000 65 1.3 / 0.95, 129 0.8 / 0.8
+//                    ELL 120,000 65 1.9 / 1.4, 97 1.3 / 1.1
+//                    BiCGSTAB 79,000 97 1.1 / 1.0, 129 0.9 / 1.0
+//   four rows:       CG 262,144 K = 33 1.8 / 1.7, 49 1.0 / 1.3; ELL 27 1.5 / 1.3, 49 0.9 / 0.9
+//                    BiCGSTAB 262,144 33 1.4 / 1.5, 49 0.8 / 1.2; ELL 27 1.2 / 1.2, 33 0.8 / 0.9
+// FP32: 1.2-3 at all of these but ELL, two rows, K = 129 0.9.  GMRES (few
+// products a step): FP64 CSR 25,000 257 1.6 / 1.4, 5,000 321 1.0, 1,000 401 0.9; the
+// others win at every K measured, to 999.
+bool pk_unstaged_worth(int solver, bool csr, bool f64, int rows, int64_t n, int64_t K) {
+  const bool bicg = solver == 1;
+  if (solver == 2) return !csr || !f64 || K <= 320;
+  if (rows == 1) return !csr || !f64 || K <= (n >= 16384 ? 320 : n > 9728 ? 160 : 0);
+  if (rows == 2) return K <= (csr ? (bicg && f64 ? 112 : 160) : f64 && n < 98304 ? 64 : 96);
+  return K <= (csr ? (bicg && f64 ? 40 : 72) : bicg && f64 ? 32 : 40);
+}
+
 // What every kernel is given: the matrix, right-hand side, x and options.
 template <typename T, typename VT>
 PkArgs<T, VT> args_of(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSpec& sp, size_t K) {
@@ -157,17 +191,23 @@ int run(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const SolveSp
   auto covers = [&](const PkShape& h) {
     return blocks_of(h) <= (h.mode == kPkCluster ? kPkCluster16 : std::min(sm_count(), kPkMaxBlocks));
   };
-  const bool published = sp.solver == 1 && sp.bj;  // no kPkFly
+  const bool f64 = sizeof(T) == 8, bicg = sp.solver == 1;
+  const bool twins = (bicg && sp.bj) || (int64_t)K > kPkFlyRow;
+  auto worth = [&](const PkShape& h, bool staged) {
+    if (h.mode == kPkCluster) return n * (int64_t)K <= (!bicg && !f64 ? kPkClusterEntriesCg32 : kPkClusterEntries);
+    return staged || pk_unstaged_worth(sp.solver, A->fmt == GKO_CSR, f64, h.rpt, n, (int64_t)K);
+  };
   auto attempt = [&](int i, bool staged) -> int {
     const PkShape& h = kPkShapes[i];
-    if (!covers(h) || (published && h.mode == kPkFly) || smem_of(h, staged) > kPkSmemMax) return GKO_NOT_SUPPORTED;
+    if (!covers(h) || (bicg && sp.bj && h.mode == kPkFly) || smem_of(h, staged) > kPkSmemMax || !worth(h, staged))
+      return GKO_NOT_SUPPORTED;
     return launch<T, VT>(A, b, x, x_zero, sp, s, out, i, staged, (int)blocks_of(h), K, smem_of(h, staged));
   };
   for (bool staged : {true, false}) {
     const int first = staged ? 0 : kPkFirstGlobal;
     for (int i = first; i <= kPkLastGlobal; ++i) {
-      if (published && staged && kPkShapes[i].mode == kPkFly) {  // its published twin
-        const int rc = attempt(i + kPkTwin, true);
+      if (twins && kPkShapes[i].mode == kPkFly) {  // its published twin
+        const int rc = attempt(i + kPkTwin, staged);
         if (rc != GKO_NOT_SUPPORTED) return rc;
       }
       const int rc = attempt(i, staged);
@@ -190,6 +230,7 @@ int run_gmres(const gko_matrix_s* A, const double* b, T* x, bool x_zero, const S
       const size_t smem = staged ? K * (size_t)rb * (sizeof(VT) + sizeof(int32_t)) : 0;
       const PkGmresKernel<T, VT> kern = pk_gmres<T, VT>(shape, staged);
       if (!kern || G > std::min(sm_count(), kPkMaxBlocks) || smem > kPkSmemMax) continue;
+      if (!staged && !pk_unstaged_worth(2, A->fmt == GKO_CSR, sizeof(T) == 8, h.rpt, n, (int64_t)K)) continue;
       if (smem > 24 * 1024)
         GKO_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPkSmemMax));
       const int64_t ld = (n + 63) / 64 * 64;

@@ -518,7 +518,7 @@ struct PkPrecond {
 // ----------------------------------------------------------------- CG --
 
 template <typename T, typename VT, int NT, int RPT, int MODE, bool ST>
-__global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
+__global__ void __launch_bounds__(NT, 1) pk_cg_kernel(PkArgs<T, VT> a) {
   constexpr bool FLY = MODE == kPkFly;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PkShared<NT, MODE> sh;
@@ -770,7 +770,7 @@ __global__ void __launch_bounds__(NT) pk_cg_kernel(PkArgs<T, VT> a) {
 // its largest norm since the last update, the change is added to x64 and r is
 // replaced by b64 - A64 x64 computed in FP64.
 template <typename T, typename VT, int NT, int RPT, int MODE, bool ST, bool REL>
-__global__ void __launch_bounds__(NT) pk_bicg_kernel(PkArgs<T, VT> a) {
+__global__ void __launch_bounds__(NT, 1) pk_bicg_kernel(PkArgs<T, VT> a) {
   constexpr bool FLY = MODE == kPkFly;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PkShared<NT, MODE> sh;
@@ -1183,14 +1183,15 @@ using PkKernel = void (*)(PkArgs<T, VT>);
 
 // Shapes: threads x rows per thread and mode, in order of preference; the
 // first that covers n (with the 16 blocks of a cluster, else one block per
-// SM) and whose entries fit is taken, so the fewest rows per SM.  Measured, us
-// per iteration (100 CG or 20 BiCGSTAB iterations, setup included), one step
+// SM) and whose entries fit is taken, so the fewest rows per SM; what long rows
+// change about that is in persist.cu.  Measured, us per iteration (100 CG or 20 BiCGSTAB iterations, setup included), one step
 // to the next shape on either side of each line:
 //   cluster -> kPkFly after 16 x 512 rows: CG on 8,100 rows 6.2 in the cluster,
 //     7.1 as 64-thread kPkFly blocks; on 4,096 rows 4.5 and 6.7
-//   kPkFly -> kPkGrid after 512 rows per block, where the extra FMAs cost as
-//     much as the exchange they save: CG on 29,791 rows 7.6 as kPkFly blocks
-//     of 256 rows, 12.5 as kPkGrid blocks of 1,024
+//   kPkFly -> kPkGrid after 512 rows per block (CG on 29,791 rows 7.6 as kPkFly
+//     blocks of 256 rows, 12.5 as kPkGrid blocks of 1,024), and for rows of
+//     more than kPkFlyRow entries, whose extra gathers cost more than the
+//     exchange they save
 //   512 threads x 2 and 4 rows above that: CG on 91,125 rows 11.6, 238,328
 //     rows 16.4 (256 threads x 4 and 8: 12.4 and 20.4)
 struct PkShape {
@@ -1199,12 +1200,15 @@ struct PkShape {
 constexpr PkShape kPkShapes[] = {
     {32, 1, kPkCluster}, {64, 1, kPkCluster}, {128, 1, kPkCluster}, {256, 1, kPkCluster}, {256, 2, kPkCluster},
     {64, 1, kPkFly}, {128, 1, kPkFly}, {256, 1, kPkFly}, {512, 1, kPkFly}, {512, 2, kPkGrid}, {512, 4, kPkGrid},
-    // BiCGSTAB with block-Jacobi, whose preconditioned directions no gatherer can recompute, instead of kPkFly
+    // instead of kPkFly where rows are long, and for BiCGSTAB with block-Jacobi, whose preconditioned directions no
+    // gatherer can recompute
     {64, 1, kPkGrid}, {128, 1, kPkGrid}, {256, 1, kPkGrid}, {512, 1, kPkGrid}};
-constexpr int kPkNShapes = sizeof(kPkShapes) / sizeof(kPkShapes[0]);
-// (unstaged variants: shapes kPkFirstGlobal to kPkLastGlobal)
-constexpr int kPkFirstGlobal = 7, kPkLastGlobal = 10;
 constexpr int kPkTwin = 6;  // from a kPkFly shape to the published one of its size
+// unstaged variants: shapes kPkFirstGlobal to kPkLastGlobal and the twins of these
+constexpr int kPkFirstGlobal = 7, kPkLastGlobal = 10;
+constexpr bool pk_unstaged(int shape) {
+  return (shape >= kPkFirstGlobal && shape <= kPkLastGlobal) || shape >= kPkFirstGlobal + kPkTwin;
+}
 
 // The kernel of a shape, with or without staging, or null; one translation
 // unit per solver and value type instantiates them (persist_*.cu).
@@ -1223,12 +1227,12 @@ PkKernel<T, VT> pk_bicg(int shape, bool staged);
 #define GKO_PK_CG(SH, NT, RPT, MODE)                                                                  \
   if (shape == SH) {                                                                                 \
     if (staged) return pk_cg_kernel<T, VT, NT, RPT, MODE, true>;                                      \
-    if constexpr (SH >= kPkFirstGlobal && SH <= kPkLastGlobal) return pk_cg_kernel<T, VT, NT, RPT, MODE, false>;             \
+    if constexpr (pk_unstaged(SH)) return pk_cg_kernel<T, VT, NT, RPT, MODE, false>;                  \
   }
 #define GKO_PK_BICG(SH, NT, RPT, MODE)                                                                \
   if (shape == SH) {                                                                                 \
     if (staged) return pk_bicg_kernel<T, VT, NT, RPT, MODE, true, sizeof(T) == 4>;                    \
-    if constexpr (SH >= kPkFirstGlobal && SH <= kPkLastGlobal) return pk_bicg_kernel<T, VT, NT, RPT, MODE, false, sizeof(T) == 4>; \
+    if constexpr (pk_unstaged(SH)) return pk_bicg_kernel<T, VT, NT, RPT, MODE, false, sizeof(T) == 4>; \
   }
 
 }  // namespace gko

@@ -8,6 +8,7 @@ PkKernel<float, __nv_bfloat16> pk_cg<float, __nv_bfloat16>(int shape, bool stage
   using T = float;
   using VT = __nv_bfloat16;
   GKO_PK_SHAPES(GKO_PK_CG)
+  GKO_PK_BLOCK_SHAPES(GKO_PK_CG)
   return nullptr;
 }
 

@@ -271,3 +271,38 @@ def test_gmres_mixed_at_any_scale_of_matrix_and_right_hand_side(gko, n, ka, kb):
         assert res.status == G.OK, res
         runs.append((res.iterations, host(xd)))
     assert runs[1][0] == runs[0][0] and np.array_equal(runs[1][1], np.ldexp(runs[0][1], kb - ka))
+
+
+# longest row K on both sides of the lines between cluster, recomputed and published vectors, entries in
+# shared memory and in the matrix, and the multi-kernel solve
+LONG_ROWS = [(2000, 17), (2000, 33), (2000, 57), (2000, 59), (4096, 15), (4096, 27), (4096, 29), (600, 265), (600, 267),
+             (12000, 131), (12000, 135), (14000, 161), (20000, 101), (20000, 321), (20000, 323), (45000, 33),
+             (45000, 35), (78000, 17), (78000, 95), (78000, 97), (100000, 65), (160000, 7), (160000, 9), (160000, 33),
+             (160000, 41)]
+
+
+@pytest.mark.parametrize("n,K", LONG_ROWS)
+@pytest.mark.parametrize("name", ["cg", "bicgstab", "gmres"])
+def test_long_rows(gko, name, n, K):
+    G = gko
+    half = K // 2
+    rng = np.random.default_rng(K)
+    cols = np.arange(n)[:, None] + np.arange(-half, half + 1)[None, :]
+    vals = np.full(cols.shape, -1.0) if name == "cg" else rng.uniform(-1, 0, cols.shape)
+    vals[:, half] = 1.5 * K
+    ok = (cols >= 0) & (cols < n)
+    rp = np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32)
+    A = I.Csr(n, n, rp, cols[ok].astype(np.int32), vals[ok], "long")
+    M = G.from_csr(A)
+    b = np.random.default_rng(1).uniform(-1, 1, n)
+    x0, r0 = O.solve({"cg": O.CG, "bicgstab": O.BICGSTAB, "gmres": O.GMRES}[name], A, b, tol=1e-12, maxit=500)
+    assert r0.status == 0
+    fn = {"cg": G.gko_solve_cg, "bicgstab": G.gko_solve_bicgstab, "gmres": G.gko_solve_gmres}[name]
+    for M in (M, G.gko_matrix_convert_to_ell(M)):
+        for precision in (G.PRECISION_F64, G.PRECISION_MIXED_F32):
+            xd = dev(np.zeros(n))
+            res = fn(M, dev(b), xd, 1e-12, 500, G.opts(precision=precision))
+            x = host(xd)
+            assert res.status == G.OK and np.linalg.norm(x - x0) <= 1e-8 * np.linalg.norm(x0), res
+            true = np.linalg.norm(b - O.spmv_csr(A, x)) / np.linalg.norm(b)
+            assert true <= 1.01e-12 and abs(true - res.rel_residual) <= 1e-13
