@@ -1289,13 +1289,13 @@ struct BatchGraph {
 };
 constexpr int kGraphIters = 16;  // iterations per replayed batch
 
-// Rows from which unpreconditioned FP64 CG sums r.r as an FP64 tree
-// (block_tree_n).  us an iteration, tree and integer sums, 7-point: 88^3 48.6
+// Rows between which unpreconditioned FP64 CG sums r.r as an FP64 tree
+// (block_tree_n); elsewhere the integer sums are as fast and more exact.  us an iteration, tree and integer sums, 7-point: 88^3 48.6
 // and 47.2, 96^3 55.3 and 55.6, 112^3 74.1 and 78.2, 128^3 95.7 and 99.5, 144^3
-// 130.5 and 137.1, 160^3 162.2 and 164.1, 256^3 the same.  With a preconditioner,
+// 130.5 and 137.1, 160^3 162.2 and 164.1, 180^3 and 256^3 the same.  With a preconditioner,
 // in FP32 and in BiCGSTAB the integer sums are the faster or the same (Jacobi,
 // 128^3: 110.0 and 107.3; BiCGSTAB within 2% either way).
-constexpr int64_t kTreeRows = 1 << 20;
+constexpr int64_t kTreeRows = 1 << 20, kTreeRowsEnd = 1 << 22;
 
 // One Krylov solve on the device.  A: matrix whose value type matches T
 // (double: F64; float: F32/BF16).  b: FP64 right-hand side; x: T vector,
@@ -1393,7 +1393,7 @@ static int krylov_core(const gko_matrix_s* A, const double* b, T* x, bool x_zero
     // programmatic serialization (PdlScope), so its dispatch overlaps the
     // drain of the one before; each waits for that one before touching memory.
     const dim3 B256(256);
-    const bool tree = sizeof(T) == 8 && n >= kTreeRows;
+    const bool tree = sizeof(T) == 8 && n >= kTreeRows && n < kTreeRowsEnd;
     auto enqueue = [&](int count) -> int {
       PdlScope pdl(true);
       for (int it = 0; it < count; ++it) {

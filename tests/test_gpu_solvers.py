@@ -381,10 +381,10 @@ def test_solver_workloads_full_size(gko, case):
         assert np.linalg.norm(x - 1.0) <= 1e-4 * np.sqrt(A.n_rows)
 
 
-@pytest.mark.parametrize("n", [(1 << 20) - 1, 1 << 20, (1 << 20) + 1])
+@pytest.mark.parametrize("n", [(1 << 20) - 1, 1 << 20, (1 << 22) - 1, 1 << 22])
 def test_cg_where_the_sums_change_form(gko, n):
-    """Unpreconditioned FP64 CG around 2^20 rows, where its block sums change
-    from integers to an FP64 tree: the oracle's iterate after 12 steps."""
+    """Unpreconditioned FP64 CG at 2^20 and 2^22 rows, between which its block
+    sums are an FP64 tree: the oracle's iterate after 12 steps."""
     G = gko
     i = np.arange(n)
     A = I.Csr(n, n, np.arange(0, 3 * n + 1, 3, dtype=np.int32)[: n + 1],
