@@ -472,7 +472,9 @@ GKO_API int gko_batch_cg(gko_batch B, const double *b, double *x, double rel_tol
  * whole batch for every schedule, warp_rows in {0, 64, 144, 256} x threads
  * per block in {256, 512, 1024} x storage CSR or ELL (solving from a scratch
  * copy of x0; x0 is not changed), keeps the fastest and reports it (outputs
- * may be NULL; best_ms in milliseconds).  Synchronises `stream`. */
+ * may be NULL; best_ms in milliseconds).  A mixed-precision batch whose systems
+ * are all solved resident (gko_batch_set_precision) keeps its schedule, which
+ * such a solve does not use.  Synchronises `stream`. */
 GKO_API int gko_batch_tune(gko_batch B, const double *b, const double *x0, double rel_tol, int32_t max_iters,
                            int32_t *warp_rows, int32_t *threads, int32_t *storage, float *best_ms, void *stream);
 

@@ -128,6 +128,24 @@ def test_batch_tuner_and_invalid_input(gko):
         G.Batch([bad])
 
 
+def test_batch_tuner_leaves_a_schedule_that_serves_no_system(gko):
+    G = gko
+    systems, bs = batch_problem(60, seed=6)
+    B = G.Batch(systems)
+    B.set_schedule(64, 512, G.BATCH_ELL)
+    B.set_precision(G.PRECISION_MIXED_F32)
+    b, x0 = dev(concat(bs)), dev(np.zeros(B.total_rows))
+    for _ in range(3):
+        t = B.tune(b, x0, 1e-10, 20000)
+        assert (t["warp_rows"], t["threads"], t["storage"]) == (64, 512, "ell") and t["ms"] > 0
+    inf = B.info()
+    assert (inf["warp_rows"], inf["threads"], inf["storage"]) == (64, 512, "ell")
+    big = G.Batch(systems + [I.laplace2d_5pt(80)])  # 6,400 rows: not resident, the search runs
+    big.set_precision(G.PRECISION_MIXED_F32)
+    t = big.tune(dev(concat(bs + [np.ones(6400)])), dev(np.zeros(big.total_rows)), 1e-10, 20000)
+    assert t["warp_rows"] in (0, 64, 144, 256) and t["ms"] > 0
+
+
 @pytest.mark.slow
 def test_batch_full_size_4096(gko):
     """The batched workload of the benchmark: 4096 systems, sides in [8, 64]."""
