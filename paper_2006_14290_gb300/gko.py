@@ -154,9 +154,13 @@ def _check(status: int, where: str):
 def _stream(stream):
     if stream is None:
         # the current stream's handle without a torch Stream object around it:
-        # 0.4 us a call instead of 3.2, of 8.8 for the smallest gko_spmv
+        # 0.4 us a call instead of 3.2, of 8.8 for the smallest gko_spmv; not a
+        # public function, so a torch without it takes the public way
         import torch
-        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return C.c_void_p(raw(torch.cuda.current_device()))
     if isinstance(stream, int):
         return C.c_void_p(stream)
     return C.c_void_p(stream.cuda_stream)

@@ -100,3 +100,20 @@ def test_product_package_does_not_reach_the_oracle():
                     src = fh.read()
                 assert not re.search(r"^\s*(import|from)\s+oracle\b", src, re.M), f
                 assert "gko_oracle" not in src and "liboracle" not in src, f
+
+
+def test_current_stream_with_and_without_the_raw_handle(monkeypatch):
+    """The default stream argument is torch's current stream, also with a
+    torch that lacks the private accessor of its handle."""
+    torch = pytest.importorskip("torch")
+
+    class Stream:
+        cuda_stream = 0x77
+
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 0x50 + device, raising=False)
+    assert G._stream(None).value == 0x53
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert G._stream(None).value == 0x77
+    assert G._stream(5).value == 5 and G._stream(Stream).value == 0x77
