@@ -1634,7 +1634,7 @@ static int map_status(int st) {
 // the column-major ELL kernel streams the operator faster than the CSR
 // kernels (7-point 128^3 FP32 SpMV 30 us vs 41 us), while in FP64 the CSR
 // row-block kernel keeps up (CG on 7-point 256^3: 302 ms CSR, 314 ms ELL).
-// Systems small enough for the single-launch CG (CSR only) keep CSR.
+// Systems small enough for the single-launch solvers keep CSR.
 constexpr double kInnerEllFill = 1.2;
 static int lowp_copy(gko_matrix A, gko_dtype to, cudaStream_t s, gko_matrix* out) {
   std::lock_guard<std::mutex> lk(A->mu);

@@ -114,8 +114,8 @@ struct SolveOut {
 // multi-kernel solvers.
 constexpr int64_t kSmallRows = 1 << 18;
 
-// One CG or BiCGSTAB solve in one cooperative launch (persist.cuh), or
-// GKO_NOT_SUPPORTED when it does not apply (the caller then takes the
+// One CG, BiCGSTAB or GMRES solve in one launch, a cluster or a cooperative grid
+// (persist.cuh, persist_gmres.cuh), or GKO_NOT_SUPPORTED when it does not apply (the caller then takes the
 // multi-kernel solve).  x: T vector (double for an FP64 matrix, else float).
 int persist_solve(const gko_matrix_s* A, const double* b, void* x, bool x_zero, const SolveSpec& sp, cudaStream_t s,
                   SolveOut* out);

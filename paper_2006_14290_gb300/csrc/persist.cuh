@@ -18,9 +18,16 @@
 //
 // Three ways to share vectors and sums (MODE):
 //  kPkCluster: one cluster of up to 16 blocks; published vectors and slots in
-//    shared memory, read through distributed shared memory.  An exchange takes
-//    about 450 cycles, against 1500 through L2 for 16 blocks on both dies and
-//    2600 for 128, but 16 SMs are all the FP64 pipes there are.
+//    shared memory, read through distributed shared memory.  A sum of one value
+//    takes 2,150 cycles over 16 blocks of 64 threads from the threads' values to
+//    the total in every block, 1,500 more for each further value; through L2
+//    3,430 for 16 blocks on both dies, 4,060 for 117 and 1,700 to 2,300 more
+//    (gko_diag_exchange).  But 16 SMs are all the FP64 pipes there are.  A partial sum
+//    in a cluster is taken by its tag, never by the barrier alone: a cluster
+//    CG that ordered untagged slots by barriers read one before it was written
+//    (FP32, two rows a thread) and stopped some inner solves after a step.
+//    What the barrier still orders are the published vectors: stored before
+//    its release, read after its acquire by volatile loads.
 //  kPkGrid, kPkFly: a cooperative grid; vectors in global memory, read with
 //    ld.global.cg (inside one launch L1 is not coherent across SMs).
 //  kPkFly: the vector an SpMV gathers is not published after it is formed,

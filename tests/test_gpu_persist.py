@@ -306,3 +306,41 @@ def test_long_rows(gko, name, n, K):
             assert res.status == G.OK and np.linalg.norm(x - x0) <= 1e-8 * np.linalg.norm(x0), res
             true = np.linalg.norm(b - O.spmv_csr(A, x)) / np.linalg.norm(b)
             assert true <= 1.01e-12 and abs(true - res.rel_residual) <= 1e-13
+
+
+def test_mixed_cluster_solves_repeat_on_concurrent_streams(gko):
+    """Mixed Jacobi-CG on 4,000-8,000 rows, whose FP32 inner solves run in one
+    cluster each with two rows a thread, 480 times on four threads and streams:
+    every solve converges in the steps and to the bits of the first."""
+    import concurrent.futures as cf
+
+    import torch
+
+    G = gko
+    systems = []
+    for n in (4097, 4913, 5000, 6000, 6859, 7001, 8000, 8192):
+        A = banded_system(n, 17, True, n)
+        A.val = A.val * np.exp(np.random.default_rng(n).uniform(-2, 2)).astype(np.float64)
+        systems.append((G.from_csr(A), dev(np.random.default_rng(n + 1).uniform(-1, 1, n))))
+    opt = G.opts(precision=G.PRECISION_MIXED_F32, preconditioner=G.PRECOND_JACOBI)
+
+    def run(M, b, stream):
+        with torch.cuda.stream(stream):
+            x = torch.zeros_like(b)
+            res = G.gko_solve_cg(M, b, x, 1e-11, 2000, opt)
+            stream.synchronize()
+        assert res.status == G.OK and res.rel_residual <= 1e-11, res
+        return res.iterations, host(x).tobytes()
+
+    torch.cuda.synchronize()
+    first = [run(M, b, torch.cuda.current_stream()) for M, b in systems]
+
+    def worker(k):
+        stream = torch.cuda.Stream()
+        for rep in range(15):
+            for i in np.random.default_rng(100 * k + rep).permutation(len(systems)):
+                assert run(*systems[i], stream) == first[i], (k, rep, i)
+
+    with cf.ThreadPoolExecutor(4) as ex:
+        for f in [ex.submit(worker, k) for k in range(4)]:
+            f.result()
