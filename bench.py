@@ -570,7 +570,9 @@ def batched_suite(G, dev, stream, oracle_cores=0, fp64_fma=None):
         fp64_fma = fp64_fma or fma_peak(G, dev)
         fp64_frac = fmas / (ms * 1e-3) / fp64_fma
         res[tag] = {"status": int(code), "time_ms": round(ms, 3), "systems_per_s": round(4096 / (ms * 1e-3), 1),
-                    "schedule": tuned, "tuned_over": "warp rows {0,64,144,256} x threads {256,512,1024} x CSR/ELL",
+                    "schedule": tuned,
+                    "tuned_over": "no schedule: every system is solved resident on an SM" if mixed
+                    else "warp rows {0,64,144,256} x threads {256,512,1024} x CSR/ELL",
                     "iterations_total": int(it.sum()), "iterations_max": int(it.max()),
                     "max_rel_residual": float(rr.max()), "bytes": nbytes, "fp64_fmas": fmas,
                     "GB_s": round(nbytes / (ms * 1e-3) / 1e9, 1),
