@@ -180,6 +180,36 @@ def traffic_record():
     return d
 
 
+LINE_MAX = 3000  # characters: what a reader of the last lines of the output still gets whole
+
+
+def summary_line(result):
+    """The JSON line on standard output: the headline and a short form of each
+    leg.  The full record (22,000 characters) goes to standard error."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "roofline", "e2e", "clocks", "gpu_launches", "cpu_baseline")
+    line = {k: result[k] for k in keys if k in result}
+    line["config"] = {k: v for k, v in result["config"].items() if k not in ("tuned_plans", "skipped")}
+    if "cpu_baseline" in line:
+        line["cpu_baseline"] = {k: v for k, v in line["cpu_baseline"].items() if k != "cores_all"}
+    solvers = result.get("solvers", {})
+    short = {k: v["time_ms"] for k, v in solvers.items() if isinstance(v, dict) and "time_ms" in v}
+    short.update({f"batch4096_{k}": v["time_ms"] for k, v in solvers.get("batched_cg", {}).items()
+                  if isinstance(v, dict) and "time_ms" in v})
+    if short:
+        line["solvers_ms"] = short
+    serving = {k: [v["converged"], v["p99_ms"], v["solves_per_s"]] for k, v in result.get("serving", {}).items()
+               if isinstance(v, dict) and "p99_ms" in v}
+    if serving:
+        line["serving_converged_p99ms_per_s"] = serving
+    line["full_record"] = "standard error"
+    for drop in ("serving_converged_p99ms_per_s", "solvers_ms"):
+        if len(json.dumps(line)) <= LINE_MAX:
+            break
+        line.pop(drop, None)
+    return json.dumps(line)
+
+
 # ----------------------------------------------------------------- solvers --
 
 def oracle_solver_sample(solver, A, b, iters, pc=False, bs=0):
@@ -1212,7 +1242,8 @@ def run_ours(args):
             result["serving"] = serving_suite(G)
         if world == 1 and not args.no_cpu_baseline:
             result["cpu_baseline"] = cpu_baseline(mats)
-        print(json.dumps(result), flush=True)
+        print(json.dumps(result), file=sys.stderr, flush=True)
+        print(summary_line(result), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
